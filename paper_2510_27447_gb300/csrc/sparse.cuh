@@ -121,10 +121,95 @@ __device__ __forceinline__ void load_descriptor(D& dst, const D* src) {
   __syncthreads();
 }
 
-// block-wide sum of NV values; result valid in thread 0
-template <int NV, class T = double>
+// Sum of NV <= 4 values over a warp, the values spread over the lanes as the
+// butterfly narrows: the step over lane bit 4 (and bit 3) leaves each half
+// (quarter) of the warp with its own value, so NV = 2 takes 5 additions and
+// NV = 4 takes 6 instead of NV x 5.  Lane l ends with value lane_value<NV>(l).
+template <int NV>
+__device__ __forceinline__ int lane_value(int lane) {
+  return NV == 1 ? 0 : NV == 2 ? lane >> 4 : lane >> 3;
+}
+template <int NV, class T>
+__device__ __forceinline__ T warp_sum_spread(const T (&v)[NV]) {
+  static_assert(NV >= 1 && NV <= 4, "up to four values");
+  const int lane = threadIdx.x & 31;
+  T x;
+  if constexpr (NV == 1) {
+    x = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
+  } else if constexpr (NV == 2) {
+    const bool hi = (lane & 16) != 0;
+    x = (hi ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[1], 16);
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
+  } else {
+    const T v3 = NV == 4 ? v[NV - 1] : T(0);
+    const bool hi = (lane & 16) != 0, hj = (lane & 8) != 0;
+    const T a = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
+    const T b = (hi ? v3 : v[1]) + __shfl_xor_sync(0xffffffffu, hi ? v[1] : v3, 16);
+    x = (hj ? b : a) + __shfl_xor_sync(0xffffffffu, hj ? a : b, 8);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// block-wide sum of NV values; result valid in thread 0.
+//
+// FP64: the SM's FP64 pipe takes two lanes a clock, so one addition of a warp
+// holds it for 16 clocks however few lanes count, and a shuffle tree over 16
+// warps (NV x 5 additions a warp) is 1280 NV clocks of pipe time.  One or two
+// values a thread therefore go through shared memory to the first four warps,
+// whose lanes all add distinct values (3 NV + 5 additions a warp for 512
+// threads); more values use the spread butterfly in every warp.  MAXT bounds
+// the block size (the FP64 staging area).  Measured against a shuffle tree in
+// every warp and a second one over all warps' partials in grid_total (FP64 step
+// of three nodes and two sweeps): LR91 65^2 6.48 -> 5.71 ms, TP06 257^2 10.28 ->
+// 9.74 ms, TP06 slab 101x101x26 34.0 -> 33.0 ms.
+template <int NV, class T = double, int MAXT = 1024>
 __device__ __forceinline__ void block_sum(T (&v)[NV], T (*sh)[32]) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if constexpr (sizeof(T) == 8) {
+    constexpr int kRed = 128;                      // threads that add
+    int nw = int(blockDim.x) >> 5;                 // warps holding a partial sum afterwards
+    if constexpr (NV <= 2) {
+      __shared__ T st[NV][MAXT];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) st[k][threadIdx.x] = v[k];
+      __syncthreads();
+      nw = nw < kRed / 32 ? nw : kRed / 32;
+      if (wid < nw) {
+        for (int t = threadIdx.x + kRed; t < int(blockDim.x); t += kRed)
+#pragma unroll
+          for (int k = 0; k < NV; ++k) v[k] += st[k][t];
+        const T x = warp_sum_spread<NV>(v);
+        if ((lane & (32 / NV - 1)) == 0) sh[lane_value<NV>(lane)][wid] = x;
+      }
+    } else {
+      const T x = warp_sum_spread<NV>(v);
+      if ((lane & 7) == 0 && lane_value<NV>(lane) < NV) sh[lane_value<NV>(lane)][wid] = x;
+    }
+    __syncthreads();
+    if (NV <= 2) {
+      if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          T x = sh[k][0];
+          for (int w = 1; w < nw; ++w) x += sh[k][w];
+          v[k] = x;
+        }
+    } else if (wid == 0) {
+      T p[NV];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) p[k] = lane < nw ? sh[k][lane] : T(0);
+      const T x = warp_sum_spread<NV>(p);
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] = __shfl_sync(0xffffffffu, x, 8 * k);
+    }
+    // one and two values: sh and st are rewritten only behind the first
+    // barrier of the next call
+    if (NV > 2) __syncthreads();
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     T x = v[k];
@@ -147,17 +232,35 @@ __device__ __forceinline__ void block_sum(T (&v)[NV], T (*sh)[32]) {
 }
 
 // every block sums part[b*STRIDE + slot] over b = 0..nb-1 in the same order
+// (FP64: by one warp, see block_sum; a device-wide barrier separates any two
+// calls, so bc is not rewritten while it is read)
 template <int NV, class T = double, int STRIDE = 4>
 __device__ __forceinline__ void grid_total(const T* part, const int (&slot)[NV], int nb, T (&out)[NV],
                                            T (*sh)[32]) {
   T v[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) v[k] = T(0);
+  __shared__ T bc[NV];
+  if constexpr (sizeof(T) == 8) {
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+#pragma unroll 4
+      for (int b = lane; b < nb; b += 32)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] += __ldcg(part + b * STRIDE + slot[k]);
+      const T x = warp_sum_spread<NV>(v);
+      constexpr int G = NV == 1 ? 32 : NV == 2 ? 16 : 8;
+      if ((lane & (G - 1)) == 0 && lane_value<NV>(lane) < NV) bc[lane_value<NV>(lane)] = x;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) out[k] = bc[k];
+    return;
+  }
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < NV; ++k) v[k] += __ldcg(part + b * STRIDE + slot[k]);
   block_sum<NV, T>(v, sh);
-  __shared__ T bc[NV];
   if (threadIdx.x == 0)
 #pragma unroll
     for (int k = 0; k < NV; ++k) bc[k] = v[k];

@@ -217,7 +217,7 @@ __device__ __forceinline__ void level_rows_m(const SellDevT<T>& A, const T* x0, 
         if (ON(0)) v[0] += a * __ldg(x0 + c);
         if (ON(1)) v[1] += a * __ldg(x1 + c);
       }
-      block_sum<2, T>(v, shb);
+      block_sum<2, T, kCsrBlockLanes>(v, shb);
       if (threadIdx.x == 0) epi(i, v);
     }
   } else if ((K & kRowsCsrLanes) && A.rp) {

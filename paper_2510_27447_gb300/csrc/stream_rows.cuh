@@ -152,7 +152,7 @@ __device__ __forceinline__ void level_rows(const SellDevT<T>& M, const T* x, boo
       T v[1] = {T(0)};
       for (int64_t p = __ldg(M.rp + i) + threadIdx.x; p < e; p += blockDim.x)
         v[0] += __ldg(M.val + p) * __ldg(x + __ldg(M.col + p));
-      block_sum<1, T>(v, shb);
+      block_sum<1, T, kCsrBlockLanes>(v, shb);
       if (threadIdx.x == 0) epi(i, v[0]);
     }
   } else if ((K & kRowsCsrLanes) && M.rp) {
@@ -237,7 +237,7 @@ __device__ __forceinline__ bool last_block_total(T (&v)[NV], void* partv, unsign
   __shared__ T tot[NV];
   __shared__ int amlast;
   T* part = static_cast<T*>(partv);
-  block_sum<NV, T>(v, sh);
+  block_sum<NV, T, kSB>(v, sh);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) part[sg.lb * NV + k] = v[k];
@@ -253,7 +253,7 @@ __device__ __forceinline__ bool last_block_total(T (&v)[NV], void* partv, unsign
   for (int b = threadIdx.x; b < sg.nb; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < NV; ++k) acc[k] += __ldcg(part + b * NV + k);
-  block_sum<NV, T>(acc, sh);
+  block_sum<NV, T, kSB>(acc, sh);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) tot[k] = acc[k];
