@@ -32,6 +32,8 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_amg_kernel(cons
   load_descriptor(sM, Mp);
   const AmgDev& M = sM;
   __shared__ double sh[4][32];
+  __shared__ double s_x, s_y;   // scalars of the block (by_one)
+  __shared__ int s_code;
   if (a.gate && *a.gate == 0) return;
   const int n = a.n;
   const int nb = gridDim.x;
@@ -60,10 +62,12 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_amg_kernel(cons
   if (!grid_barrier(a.bar, nb, a.status)) return;
   double tot[2];
   grid_total<2>(a.part, {0, 1}, nb, tot, sh);
-  const double mean_b = a.project ? tot[0] / double(n) : 0.0;
-  double bb = a.project ? tot[1] - double(n) * mean_b * mean_b : tot[1];
-  if (bb < 0.0) bb = 0.0;
-  const double tol2 = a.tol * a.tol * bb;
+  by_one([&] {
+    s_x = a.project ? tot[0] / double(n) : 0.0;
+    const double bb = a.project ? tot[1] - double(n) * s_x * s_x : tot[1];
+    s_y = a.tol * a.tol * (bb < 0.0 ? 0.0 : bb);
+  });
+  const double mean_b = s_x, tol2 = s_y;
   double rr_loc = 0.0;
   for (int i = i0; i < n; i += stride) {
     const double r = a.r[i] - mean_b;
@@ -80,11 +84,11 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_amg_kernel(cons
   }
   if (!grid_barrier(a.bar, nb, a.status)) return;
   grid_total<2>(a.part, {2, 3}, nb, tot, sh);
-  double rho = tot[0];
-  double rr = tot[1];
+  double rho = tot[0];   // kept by thread 0 from here on
 
   int it = 0, fail = 0;
-  bool done = !(rr > tol2);
+  by_one([&] { s_code = !(tot[1] > tol2) ? 1 : 0; });
+  const bool done = s_code != 0;
   double beta = 0.0;
   while (!done) {
     double pq[1] = {0.0};
@@ -102,11 +106,15 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_amg_kernel(cons
     if (!grid_barrier(a.bar, nb, a.status)) return;
     double t1[1];
     grid_total<1>(a.part, {0}, nb, t1, sh);
-    if (!(t1[0] > 0.0)) {
-      fail = isfinite(t1[0]) ? ST_INDEFINITE : ST_NONFINITE;
+    by_one([&] {
+      s_code = t1[0] > 0.0 ? 0 : isfinite(t1[0]) ? ST_INDEFINITE : ST_NONFINITE;
+      s_x = rho / t1[0];
+    });
+    if (s_code != 0) {
+      fail = s_code;
       break;
     }
-    const double alpha = rho / t1[0];
+    const double alpha = s_x;
     double rrl = 0.0;
     for (int i = i0; i < n; i += stride) {
       a.x[i] += alpha * a.p[i];
@@ -125,18 +133,19 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_amg_kernel(cons
     if (!grid_barrier(a.bar, nb, a.status)) return;
     grid_total<2>(a.part, {2, 3}, nb, tot, sh);
     ++it;
-    rr = tot[1];
-    if (!isfinite(rr) || !isfinite(tot[0])) {
-      fail = ST_NONFINITE;
+    by_one([&] {
+      s_code = !isfinite(tot[1]) || !isfinite(tot[0]) ? ST_NONFINITE
+               : tot[1] <= tol2                       ? -1
+               : it >= a.maxit                        ? ST_NOT_CONVERGED
+                                                      : 0;
+      s_y = tot[0] / rho;
+      rho = tot[0];
+    });
+    if (s_code != 0) {
+      fail = s_code > 0 ? s_code : 0;
       break;
     }
-    if (rr <= tol2) break;
-    if (it >= a.maxit) {
-      fail = ST_NOT_CONVERGED;
-      break;
-    }
-    beta = tot[0] / rho;
-    rho = tot[0];
+    beta = s_y;
   }
 
   if (a.pin >= 0) {
@@ -151,7 +160,8 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_amg_kernel(cons
     if (!grid_barrier(a.bar, nb, a.status)) return;
     double t1[1];
     grid_total<1>(a.part, {0}, nb, t1, sh);
-    const double mean = t1[0] / double(n);
+    by_one([&] { s_x = t1[0] / double(n); });
+    const double mean = s_x;
     for (int i = i0; i < n; i += stride) a.x[i] -= mean;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {

@@ -34,6 +34,8 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed_kernel(const __grid_const
   const AmgDevF& M = sM;
   __shared__ double shd[4][32];
   __shared__ float shf[4][32];
+  __shared__ double s_d[6];     // FP64 scalars of the block (by_one)
+  __shared__ int s_code;
   if (a.gate && *a.gate == 0) return;
   const int n = a.n;
   const int nb = gridDim.x;
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed_kernel(const __grid_const
     m.b64[i] = b;
     double d = a.valA[a.diagpos[i]];
     if (a.dextra) d += a.dextra[i];
-    m.invd32[i] = float(1.0 / d);
+    m.invd32[i] = 1.0f / float(d);
     acc0[0] += b;
     acc0[1] += b * b;
     if (fused) {
@@ -87,10 +89,13 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed_kernel(const __grid_const
     tot[0] = t01[0];
     tot[1] = t01[1];
   }
-  const double mean_b = a.project ? tot[0] / double(n) : 0.0;
-  double bb = a.project ? tot[1] - double(n) * mean_b * mean_b : tot[1];
-  if (bb < 0.0) bb = 0.0;
-  const double tol2 = a.tol * a.tol * bb;
+  by_one([&] {
+    s_d[0] = a.project ? tot[0] / double(n) : 0.0;
+    const double bb = a.project ? tot[1] - double(n) * s_d[0] * s_d[0] : tot[1];
+    s_d[1] = bb < 0.0 ? 0.0 : bb;
+    s_d[2] = a.tol * a.tol * s_d[1];
+  });
+  const double mean_b = s_d[0], bb = s_d[1], tol2 = s_d[2];
   if (a.project)
     for (int i = i0; i < n; i += stride) m.b64[i] -= mean_b;
 
@@ -124,27 +129,32 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed_kernel(const __grid_const
       grid_total<1, double>(a.part, {2}, nb, t1, shd);
       rr64 = t1[0];
     }
-    if (!isfinite(rr64)) {
-      fail = ST_NONFINITE;
-      break;
-    }
-    if (m.max_outer > 1 && rr64 <= tol2) break;
-    if (outer >= m.max_outer) {
-      if (m.max_outer > 1) fail = ST_NOT_CONVERGED;
-      break;
-    }
-    if (!(rr64 > 0.0)) break;   // b = 0 with x = 0
     // the inner system is scaled to a unit residual (FP32 range is then never
     // an issue, whatever the magnitude of b) and solved until its residual is
     // tol_inner, or just what the outer tolerance still needs
-    const double scale = sqrt(rr64);
-    const double inv_scale = 1.0 / scale;
-    double tgt = double(m.tol_inner) * double(m.tol_inner);
-    if (m.max_outer > 1) tgt = fmax(tgt, 0.25 * tol2 / rr64);
-    // single solve: the target is tol_inner |b|, so a warm start that already
-    // reduced the residual needs fewer iterations (cold: rr64 = |b|^2)
-    else if (a.warm) tgt = fmax(tgt, tgt * bb / rr64);
-    const float target2 = float(tgt);
+    by_one([&] {
+      s_code = !isfinite(rr64)                       ? 1
+               : m.max_outer > 1 && rr64 <= tol2     ? 2
+               : outer >= m.max_outer                ? 3
+               : !(rr64 > 0.0)                       ? 2     // b = 0 with x = 0
+                                                     : 0;
+      const double scale = sqrt(rr64);
+      double tgt = double(m.tol_inner) * double(m.tol_inner);
+      if (m.max_outer > 1) tgt = fmax(tgt, 0.25 * tol2 / rr64);
+      // single solve: the target is tol_inner |b|, so a warm start that already
+      // reduced the residual needs fewer iterations (cold: rr64 = |b|^2)
+      else if (a.warm) tgt = fmax(tgt, tgt * bb / rr64);
+      s_d[3] = scale;
+      s_d[4] = 1.0 / scale;
+      s_d[5] = tgt;
+    });
+    if (s_code != 0) {
+      if (s_code == 1) fail = ST_NONFINITE;
+      if (s_code == 3 && m.max_outer > 1) fail = ST_NOT_CONVERGED;
+      break;
+    }
+    const double scale = s_d[3], inv_scale = s_d[4];
+    const float target2 = float(s_d[5]);
 
     // ---- FP32 inner CG on A d = r / |r| ----------------------------------
     for (int i = i0; i < n; i += stride) {
@@ -351,7 +361,8 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed_kernel(const __grid_const
     if (!grid_barrier(a.bar, nb, a.status)) return;
     double tm[1];
     grid_total<1, double>(a.part, {0}, nb, tm, shd);
-    const double mean = tm[0] / double(n);
+    by_one([&] { s_d[0] = tm[0] / double(n); });
+    const double mean = s_d[0];
     for (int i = i0; i < n; i += stride) a.x[i] -= mean;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -383,6 +394,8 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed2_kernel(const __grid_cons
   const AmgDevF& H1 = sH1;
   __shared__ double shd[4][32];
   __shared__ float shf[4][32];
+  __shared__ double s_d[4][2];  // FP64 scalars of the block (by_one)
+  __shared__ int s_code[2];
   if (a.gate && *a.gate == 0) return;
   const int n = a.n;
   const int nb = gridDim.x;
@@ -427,15 +440,20 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed2_kernel(const __grid_cons
     grid_total<4, double, 8>(partd, {0, 1, 2, 3}, nb, t, shd);
     for (int k = 0; k < 4; ++k) acc0[k] = t[k];
   }
-  double tol2[2];
-  for (int k = 0; k < 2; ++k) {
-    const double mean_b = a.project ? acc0[2 * k] / double(n) : 0.0;
-    double bb = a.project ? acc0[2 * k + 1] - double(n) * mean_b * mean_b : acc0[2 * k + 1];
-    if (bb < 0.0) bb = 0.0;
-    tol2[k] = a.tol * a.tol * bb;
-    if (a.project)
+  by_one([&] {
+    for (int k = 0; k < 2; ++k) {
+      const double mean_b = a.project ? acc0[2 * k] / double(n) : 0.0;
+      const double bb = a.project ? acc0[2 * k + 1] - double(n) * mean_b * mean_b : acc0[2 * k + 1];
+      s_d[0][k] = mean_b;
+      s_d[1][k] = a.tol * a.tol * (bb < 0.0 ? 0.0 : bb);
+    }
+  });
+  const double tol2[2] = {s_d[1][0], s_d[1][1]};
+  if (a.project)
+    for (int k = 0; k < 2; ++k) {
+      const double mean_b = s_d[0][k];
       for (int i = i0; i < n; i += stride) b64[k][i] -= mean_b;
-  }
+    }
 
   int fail = 0;
   long long inner_total[2] = {0, 0};
@@ -466,32 +484,35 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed2_kernel(const __grid_cons
     if (!grid_barrier(a.bar, nb, a.status)) return;
     double rr64[2];
     grid_total<2, double, 8>(partd, {4, 5}, nb, rr64, shd);
-    if (!isfinite(rr64[0]) || !isfinite(rr64[1])) {
+    by_one([&] {
+      for (int k = 0; k < 2; ++k) {
+        s_code[k] = !isfinite(rr64[k]) ? 2 : rr64[k] > tol2[k] && rr64[k] > 0.0 ? 1 : 0;
+        const double scale = s_code[k] == 1 ? sqrt(rr64[k]) : 1.0;
+        const double tgt = double(m.tol_inner) * double(m.tol_inner);
+        s_d[1][k] = scale;
+        s_d[2][k] = 1.0 / scale;
+        s_d[3][k] = s_code[k] == 1 ? fmax(tgt, 0.25 * tol2[k] / rr64[k]) : 0.0;
+      }
+    });
+    if (s_code[0] == 2 || s_code[1] == 2) {
       fail = ST_NONFINITE;
       break;
     }
-    bool active[2];
-    for (int k = 0; k < 2; ++k) active[k] = rr64[k] > tol2[k] && rr64[k] > 0.0;
+    const bool active[2] = {s_code[0] == 1, s_code[1] == 1};
     if (!active[0] && !active[1]) break;
     if (outer >= m.max_outer) {
       fail = ST_NOT_CONVERGED;
       break;
     }
-    double scale[2] = {1.0, 1.0};
-    float target2[2] = {0.0f, 0.0f};
-    for (int k = 0; k < 2; ++k)
-      if (active[k]) {
-        scale[k] = sqrt(rr64[k]);
-        double tgt = double(m.tol_inner) * double(m.tol_inner);
-        tgt = fmax(tgt, 0.25 * tol2[k] / rr64[k]);
-        target2[k] = float(tgt);
-      }
+    const double scale[2] = {s_d[1][0], s_d[1][1]};
+    const double inv_scale[2] = {s_d[2][0], s_d[2][1]};
+    const float target2[2] = {float(s_d[3][0]), float(s_d[3][1])};
 
     // ---- FP32 inner CG on both unit-scaled systems ---------------------------
     for (int i = i0; i < n; i += stride) {
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        r32[k][i] = active[k] ? float(r64[k][i] / scale[k]) : 0.0f;
+        r32[k][i] = active[k] ? float(r64[k][i] * inv_scale[k]) : 0.0f;
         d32[k][i] = 0.0f;
       }
     }
@@ -624,9 +645,14 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed2_kernel(const __grid_cons
     if (!grid_barrier(a.bar, nb, a.status)) return;
     double tm[2];
     grid_total<2, double, 8>(partd, {0, 1}, nb, tm, shd);
+    by_one([&] {
+      s_d[0][0] = tm[0] / double(n);
+      s_d[0][1] = tm[1] / double(n);
+    });
+    const double m0 = s_d[0][0], m1 = s_d[0][1];
     for (int i = i0; i < n; i += stride) {
-      X[0][i] -= tm[0] / double(n);
-      X[1][i] -= tm[1] / double(n);
+      X[0][i] -= m0;
+      X[1][i] -= m1;
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {

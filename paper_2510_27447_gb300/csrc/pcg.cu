@@ -32,6 +32,8 @@ namespace {
 template <int WMAX, int TPB>
 __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_kernel(const __grid_constant__ PcgLaunch a) {
   __shared__ double sh[4][32];
+  __shared__ double s_x, s_y;           // scalars of the block (by_one)
+  __shared__ int s_code;
   if (a.gate && *a.gate == 0) return;   // same value for every block: all skip together
   const int n = a.n;
   const int nb = gridDim.x;
@@ -88,10 +90,12 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_kernel(const __
     tot[0] = t01[0];
     tot[1] = t01[1];
   }
-  const double mean_b = a.project ? tot[0] / double(n) : 0.0;
-  double bb = a.project ? tot[1] - double(n) * mean_b * mean_b : tot[1];
-  if (bb < 0.0) bb = 0.0;
-  const double tol2 = a.tol * a.tol * bb;
+  by_one([&] {
+    s_x = a.project ? tot[0] / double(n) : 0.0;
+    const double bb = a.project ? tot[1] - double(n) * s_x * s_x : tot[1];
+    s_y = a.tol * a.tol * (bb < 0.0 ? 0.0 : bb);
+  });
+  const double mean_b = s_x, tol2 = s_y;
 
   // ---- phase 1: z = D^-1 r, p = z (projected systems) ---------------------
   if (!fused) {
@@ -115,12 +119,12 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_kernel(const __
     tot[2] = t23[0];
     tot[3] = t23[1];
   }
-  double rho = tot[2];
-  double rr = tot[3];
+  double rho = tot[2];           // kept by thread 0 from here on
 
   int it = 0;
   int fail = 0;
-  bool done = !(rr > tol2);      // includes b = 0
+  by_one([&] { s_code = !(tot[3] > tol2) ? 1 : 0; });   // includes b = 0
+  const bool done = s_code != 0;
   double beta = 0.0;
   while (!done) {
     // phase A
@@ -140,11 +144,15 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_kernel(const __
     if (!grid_barrier(a.bar, nb, a.status)) return;
     double t1[1];
     grid_total<1>(a.part, {0}, nb, t1, sh);
-    if (!(t1[0] > 0.0)) {
-      fail = isfinite(t1[0]) ? ST_INDEFINITE : ST_NONFINITE;
+    by_one([&] {
+      s_code = t1[0] > 0.0 ? 0 : isfinite(t1[0]) ? ST_INDEFINITE : ST_NONFINITE;
+      s_x = rho / t1[0];
+    });
+    if (s_code != 0) {
+      fail = s_code;
       break;
     }
-    const double alpha = rho / t1[0];
+    const double alpha = s_x;
     // phase B
     double acc[2] = {0.0, 0.0};
     for (int i = i0; i < n; i += stride) {
@@ -165,18 +173,16 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_kernel(const __
     double tk[2];
     grid_total<2>(a.part, {2, 3}, nb, tk, sh);
     ++it;
-    rr = tk[1];
-    if (!isfinite(rr)) {
-      fail = ST_NONFINITE;
+    by_one([&] {
+      s_code = !isfinite(tk[1]) ? ST_NONFINITE : tk[1] <= tol2 ? -1 : it >= a.maxit ? ST_NOT_CONVERGED : 0;
+      s_y = tk[0] / rho;
+      rho = tk[0];
+    });
+    if (s_code != 0) {
+      fail = s_code > 0 ? s_code : 0;
       break;
     }
-    if (rr <= tol2) break;
-    if (it >= a.maxit) {
-      fail = ST_NOT_CONVERGED;
-      break;
-    }
-    beta = tk[0] / rho;
-    rho = tk[0];
+    beta = s_y;
   }
 
   // ---- normalisation of the singular elliptic solution ----------------------
@@ -192,7 +198,8 @@ __global__ void __launch_bounds__(TPB, BD_SOLVER_MIN_BLOCKS) pcg_kernel(const __
     if (!grid_barrier(a.bar, nb, a.status)) return;
     double t1[1];
     grid_total<1>(a.part, {0}, nb, t1, sh);
-    const double mean = t1[0] / double(n);
+    by_one([&] { s_x = t1[0] / double(n); });
+    const double mean = s_x;
     for (int i = i0; i < n; i += stride) a.x[i] -= mean;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {

@@ -270,6 +270,21 @@ __device__ __forceinline__ void grid_total(const T* part, const int (&slot)[NV],
   __syncthreads();
 }
 
+// FP64 scalars of a Krylov loop (divisions, square roots, comparisons), formed
+// by one thread for the whole block: a scalar instruction that every warp
+// executes holds the FP64 pipe for 16 clocks a warp, a division in 16 warps
+// for some 3,000.  f runs in thread 0 and writes shared variables that the
+// block reads after the call; a barrier lies between those reads and the next
+// call (a block sum or a device-wide barrier).  Measured, step times before /
+// after: LR91 bath sheet 401^2 mixed 5.26 / 4.93 ms, LR91 513^2 mixed 9.46 /
+// 9.13, TP06 257^2 mixed 3.18 / 3.09 and FP64 9.89 / 9.53, slab 101x101x26
+// FP64 33.0 / 32.1.
+template <class F>
+__device__ __forceinline__ void by_one(F&& f) {
+  if (threadIdx.x == 0) f();
+  __syncthreads();
+}
+
 // sum_k val[k] x[col[k]] over row i of a SELL-32 operator.  For WMAX > 0 the
 // loads are fully unrolled and predicated so a thread issues all its column
 // and value loads back to back (memory-level parallelism); WMAX = 0 loops.
