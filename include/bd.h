@@ -92,7 +92,13 @@ typedef struct {
   double sbath;
 } bd_cond_t;
 
-/* Options; bd_default_options() fills every field. */
+/* Options; bd_default_options() fills every field.
+ *
+ * Small meshes whose cg_block, cg_grid, cg_cluster, solver_tier and streaming
+ * are the defaults solve in one thread-block cluster, with operators, hierarchy
+ * and vectors in its shared memory (up to about 19,000 nodes of a triangle mesh in
+ * mixed precision, 13,000 in FP64); setting one of these options asks for the
+ * grid-wide kernels it configures. */
 typedef struct {
   int precision;         /* bd_precision_t */
   int mass_lumped;       /* 1: lumped mass also on dv/dt (default 0: consistent) */
@@ -110,8 +116,10 @@ typedef struct {
   double spd_margin;     /* condensed-diagonal safeguard factor (default 0.9, 0 disables) */
   int use_graph;         /* 1: capture each step shape into a CUDA graph and replay it (default 1) */
   int elliptic_precond;  /* 1: aggregation AMG V(1,1) cycle (default; meshes small enough
-                            for the dense coarse level use Jacobi), 0: Jacobi */
-  int amg_coarse_max;    /* rows of the dense coarsest AMG level (0 = default 1500) */
+                            for the dense coarse level use Jacobi, but mixed-precision
+                            cluster solves of them a hierarchy of their own), 0: Jacobi */
+  int amg_coarse_max;    /* rows of the dense coarsest AMG level (0 = default 1500; 384 in
+                            cluster solves) */
   int cg_block;          /* CG threads per block (0 = auto: 512) */
   int cg_grid;           /* CG blocks (0 = auto: one per cg_block rows, at most the co-resident maximum) */
   /* device memory hooks (NULL => cudaMalloc/cudaFree); ctx is passed back.  Blocks

@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "bd_internal.h"
+#include "resident.h"
 
 namespace bd {
 cudaError_t launch_eval(int model, int precision, int64_t n, const double* X, const double* istim, double inv_cm,
@@ -159,6 +160,14 @@ struct bd_state {
   double* spart = nullptr;
   double *sb64 = nullptr, *sr64 = nullptr;
   double *sr = nullptr, *sz = nullptr, *sp = nullptr, *sq = nullptr, *sd = nullptr, *sinvd = nullptr;
+  // cluster-resident solves (resident.cu): plan and device copies; res_on: every
+  // solve of this handle takes them
+  bool res_on = false;
+  bool res_amg = false;           // the elliptic solves have a hierarchy
+  ResShape res;
+  ResCta* res_cta = nullptr;
+  unsigned char *res_g0 = nullptr, *res_gA = nullptr;
+  void* res_cinv = nullptr;
   int s64_sys = 1;                // systems the FP64 workspaces above (but sinvd) hold
   cudaStream_t side[2] = {nullptr, nullptr};
   int pcg_grid = 1, pcg_block = 512, pcg_max = 1;
@@ -368,6 +377,94 @@ PcgLaunch pcg_base(bd_state* s) {
   return P;
 }
 
+// a cluster-resident solve over the first n rows; amg: with the hierarchy
+ResLaunch res_base(bd_state* s, int n, bool amg) {
+  const ResShape& R = s->res;
+  ResLaunch A{};
+  A.n = n;
+  A.N = int(s->N);
+  A.q0 = R.q0;
+  A.C = R.C;
+  A.off_lcol = R.off_lcol;
+  A.off_push = R.off_push;
+  A.img0 = R.img0;
+  A.slots0 = R.slots0;
+  A.nent_max = R.nent_max;
+  A.cta = s->res_cta;
+  A.g0 = s->res_g0;
+  if (amg) {
+    A.imgA = R.imgA[s->precision == BD_MIXED ? 0 : 1];
+    A.gA = s->res_gA;
+    A.cinv = s->res_cinv;
+    A.nlev = R.nlev;
+    A.nc = R.nc;
+    A.ldc = R.ldc;
+    for (int l = 0; l < kResLevels; ++l) {
+      A.slotsL[l] = R.slotsL[l];
+      A.qL[l] = R.qL[l];
+    }
+    A.use_amg = 1;
+  }
+  A.sptr = s->sptr;
+  A.swidth = s->swidth;
+  A.col = s->col;
+  A.diagpos = s->diagpos;
+  A.status = s->d_status;
+  A.gate = s->opts.sweep_tol > 0 ? s->gate : nullptr;
+  A.pin = -2;
+  return A;
+}
+
+ResLaunch res_elliptic(bd_state* s, const double* v, double* u) {
+  const bool mixed = s->precision == BD_MIXED;
+  ResLaunch A = res_base(s, int(s->N), s->res_amg);
+  A.valA = s->Aie;
+  A.valT = mixed ? static_cast<const void*>(s->fAie) : static_cast<const void*>(s->Aie);
+  A.val1 = s->Ai;
+  A.va = v;
+  A.c1 = -1.0;
+  A.project = 1;
+  A.warm = 1;
+  A.x = u;
+  A.pin = s->opts.pin_node >= 0 ? s->opts.pin_node : -1;
+  A.max_outer = mixed ? 12 : 1;
+  A.inner_cap = s->opts.cg_cap_e;
+  A.tol = s->opts.cg_tol_e;
+  A.tol_inner = BD_MIXED_TOL_INNER;
+  A.iters_acc = s->d_stats + 0;
+  A.solves_acc = s->d_stats + 1;
+  A.outer_acc = s->d_stats + 4;
+  return A;
+}
+
+ResLaunch res_parabolic(bd_state* s, double alpha, double c1, const double* va, double c2, const double* vb, double* x,
+                        bool node_terms, bool warm) {
+  const bool mixed = s->precision == BD_MIXED;
+  ResLaunch A = res_base(s, int(s->NT), false);   // tissue rows; their bath columns hold zeros
+  A.valA = p_values(s, alpha);
+  A.valT = mixed ? static_cast<const void*>(p_values_f(s, alpha)) : static_cast<const void*>(A.valA);
+  A.dextra = node_terms ? s->dgs : nullptr;
+  A.rl = node_terms ? s->rl : nullptr;
+  A.val1 = s->Ai;
+  A.va = va;
+  A.c1 = c1;
+  if (vb) {
+    A.val2 = s->Mv;
+    A.vb = vb;
+    A.c2 = c2;
+  }
+  A.warm = warm ? 1 : 0;
+  A.x = x;
+  A.max_outer = 1;
+  A.inner_cap = s->opts.cg_cap_p;
+  A.tol = s->opts.cg_tol_p;
+  A.tol_inner = mixed ? std::max(s->opts.cg_tol_p, 1e-6) : s->opts.cg_tol_p;
+  A.iters_acc = s->d_stats + 2;
+  A.solves_acc = s->d_stats + 3;
+  A.outer_acc = s->d_stats + 5;
+  return A;
+}
+
 // the SELL-32/4 copy (values val4) of a launch's FP32 operator, when the
 // handle keeps one
 void set_vec4(const bd_state* s, StreamLaunch& A, const float* val4) {
@@ -460,6 +557,12 @@ int elliptic(bd_state* s, const double* v, double* u) {
     CK(launch_copy(s->NT, v, s->vfull, s->stream, P.gate));
     v = s->vfull;
   }
+  if (s->res_on) {
+    const ResLaunch A = res_elliptic(s, v, u);
+    Timed t(s, BD_K_PCG_ELLIPTIC);
+    CK(res_solve(s->res, s->precision == BD_MIXED, s->res_amg, &A, 1, nullptr, 0, s->stream));
+    return BD_OK;
+  }
   P.valA = s->Aie;
   P.val1 = s->Ai;
   P.va = v;
@@ -496,6 +599,20 @@ int elliptic(bd_state* s, const double* v, double* u) {
 // two solves
 int elliptic2(bd_state* s, const double* v1, double* u1, const double* v2, double* u2) {
   const bool mixed = s->precision == BD_MIXED;
+  if (s->res_on) {   // two clusters of one launch
+    if (s->NT < s->N) {
+      Timed t(s, BD_K_COMBINE, 2);
+      const int* gate = s->opts.sweep_tol > 0 ? s->gate : nullptr;
+      CK(launch_copy(s->NT, v1, s->vfull, s->stream, gate));
+      CK(launch_copy(s->NT, v2, s->vfull2, s->stream, gate));
+      v1 = s->vfull;
+      v2 = s->vfull2;
+    }
+    const ResLaunch A[2] = {res_elliptic(s, v1, u1), res_elliptic(s, v2, u2)};
+    Timed t(s, BD_K_PCG_ELLIPTIC);
+    CK(res_solve(s->res, mixed, s->res_amg, A, 2, nullptr, 0, s->stream));
+    return BD_OK;
+  }
   // pairs: mixed AMG solves in both forms, FP64 AMG solves in the streaming form
   const bool pair = s->use_amg && s->opts.pair_solve >= 0 && (mixed ? s->two_rhs : s->streaming && s->pair64);
   if (!pair) {
@@ -561,6 +678,12 @@ int elliptic2(bd_state* s, const double* v1, double* u1, const double* v2, doubl
 // false drops diag(dgs) and rl (the plain Crank-Nicolson operator)
 int parabolic(bd_state* s, double alpha, double c1, const double* va, double c2, const double* vb, double* x,
               bool node_terms = true, bool warm = false) {
+  if (s->res_on) {
+    const ResLaunch A = res_parabolic(s, alpha, c1, va, c2, vb, x, node_terms, warm);
+    Timed t(s, BD_K_PCG_PARABOLIC);
+    CK(res_solve(s->res, s->precision == BD_MIXED, false, &A, 1, nullptr, 0, s->stream));
+    return BD_OK;
+  }
   if (s->streaming) {
     StreamLaunch A = stream_base(s, int(s->NT));   // tissue rows; their bath columns hold zeros
     const bool mixed = s->precision == BD_MIXED;
@@ -688,19 +811,97 @@ int prepare_step(bd_state* s, double dt, int M) {
   return BD_OK;
 }
 
-// build the AMG hierarchy of A_ie on the host and upload it (SELL-32 operators)
-int setup_amg(bd_state* s, const HostOps& H) {
+HCsr elliptic_csr(const bd_state* s, const HostOps& H) {
   HCsr A;
   A.n = A.m = s->N;
   A.rp.assign(H.rowptr.begin(), H.rowptr.end());
   A.ci = H.col;
   A.v = H.Aie;
-  AmgHost AH;
+  return A;
+}
+
+// may the handle's solves be cluster-resident?  Small problems whose solver
+// options are the defaults (forced tiers, grids, clusters and the streaming
+// form ask for the other kernels).  The plan decides whether it fits; an
+// operator of more than 60 KB a block never does (hierarchy, halos and vectors
+// take three times as much), which saves building its hierarchy for nothing.
+bool res_wanted(const bd_state* s) {
+  const int64_t entry = s->precision == BD_MIXED ? 6 : 10;   // value and 16-bit column
+  return !s->streaming && s->opts.cg_cluster == 0 && s->opts.solver_tier == 0 && s->opts.cg_block == 0 &&
+         s->opts.cg_grid == 0 && s->nnz * entry <= int64_t(kResMaxCluster) * 60 * 1024;
+}
+
+// Plan and upload the cluster-resident solves and leave their hierarchy in AH
+// (*built: it is); res_on stays false when the problem does not fit.
+// Hierarchy: coarsened to kResCoarseMax rows instead of AmgParams' 1500 (the
+// dense level's product runs on 16 SMs); in mixed precision also for meshes of
+// fewer than 1500 rows.  FP64 solves of those keep Jacobi: the tolerance bounds
+// the residual, and another preconditioner would move u by as much as it allows
+// (1e-9 of u at the default 1e-10).
+int setup_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sptr, const std::vector<int>& sw,
+                   AmgHost* AH, bool* built) {
+  *built = false;
+  if (!res_wanted(s)) return BD_OK;
+  const bool mixed = s->precision == BD_MIXED;
+  AmgParams prm;
+  if (s->opts.amg_coarse_max > 0) prm.coarse_max = s->opts.amg_coarse_max;
+  else if (mixed || s->N > prm.coarse_max) prm.coarse_max = kResCoarseMax;
+  if (s->opts.elliptic_precond == 1) {
+    std::string err;
+    const int rc = amg_build(elliptic_csr(s, H), prm, AH, &err);
+    if (rc != BD_OK) return fail(s, rc, "%s", err.c_str());
+  }
+  const AmgHost* hier = s->opts.elliptic_precond == 1 && !AH->lev.empty() ? AH : nullptr;
+  // the largest cluster the device schedules: measured (ms per step, 16 / 8
+  // blocks), LR91 65^2 FP64 2.07 / 2.64, TP06 129^2 mixed 1.85 / 2.37 (8 blocks do
+  // not hold it), LR91 33^2 mixed 0.68 / 0.69
+  ResPlan P;
+  bool fits = false;
+  for (int C = kResMaxCluster; C >= 8 && !fits; C /= 2)
+    fits = res_plan_build(C, s->N, H.rowptr.data(), H.col.data(), sptr.data(), sw.data(), hier, mixed, !mixed, &P) &&
+           res_prepare(P.s, mixed, false) && (!hier || res_prepare(P.s, mixed, true));
+  if (!fits) return BD_OK;
+  auto upload = [&](const void* h, size_t bytes) -> void* {
+    void* d = dalloc(s, bytes);
+    if (d && cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, s->stream) != cudaSuccess) return nullptr;
+    return d;
+  };
+  s->res = P.s;
+  s->res_cta = static_cast<ResCta*>(upload(P.cta.data(), P.cta.size() * sizeof(ResCta)));
+  s->res_g0 = static_cast<unsigned char*>(upload(P.img0.data(), P.img0.size()));
+  bool ok = s->res_cta && s->res_g0;
+  std::vector<float> ci32;
+  if (ok && hier) {
+    const std::vector<unsigned char>& im = mixed ? P.imgA32 : P.imgA64;
+    s->res_gA = static_cast<unsigned char*>(upload(im.data(), im.size()));
+    if (mixed) ci32.assign(P.cinv.begin(), P.cinv.end());
+    s->res_cinv = mixed ? upload(ci32.data(), ci32.size() * 4) : upload(P.cinv.data(), P.cinv.size() * 8);
+    ok = s->res_gA && s->res_cinv;
+  }
+  // a bath mesh's second system gathers its potential over all nodes too
+  if (ok && s->NT < s->N && !s->vfull2)
+    ok = alloc_n(s, &s->vfull2, s->N) && cudaMemsetAsync(s->vfull2, 0, s->N * 8, s->stream) == cudaSuccess;
+  // the plan's host arrays end here
+  if (!ok || cudaStreamSynchronize(s->stream) != cudaSuccess) return fail(s, BD_ERR_OOM, "device allocation failed");
+  s->res_amg = hier != nullptr;
+  s->res_on = true;
+  *built = true;
+  return BD_OK;
+}
+
+// build the AMG hierarchy of A_ie on the host and upload it (SELL-32 operators)
+// (built: AH holds the hierarchy of the cluster-resident solves, kept for meshes
+// that have one here too)
+int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH, bool built) {
   std::string err;
   AmgParams prm;
   if (s->opts.amg_coarse_max > 0) prm.coarse_max = s->opts.amg_coarse_max;
-  const int rc = amg_build(A, prm, &AH, &err);
-  if (rc != BD_OK) return fail(s, rc, "%s", err.c_str());
+  if (s->N <= prm.coarse_max) return BD_OK;   // small operator: Jacobi-PCG is used
+  if (!built) {
+    AH = AmgHost{};
+    const int rc = amg_build(elliptic_csr(s, H), prm, &AH, &err);
+    if (rc != BD_OK) return fail(s, rc, "%s", err.c_str());
+  }
   if (AH.lev.empty()) return BD_OK;   // small operator: Jacobi-PCG is used
   if (int(AH.lev.size()) > kMaxAmgLevels)
     return fail(s, BD_ERR_ARG, "AMG hierarchy has %d levels", int(AH.lev.size()));
@@ -1233,6 +1434,7 @@ struct BatchPlan {
   std::vector<bd_state*> m;
   cudaStream_t side[2] = {nullptr, nullptr};
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};   // launches side by side within a capture
   BatchCtl* ctl = nullptr;
   // arena chunks (one per captured step shape; graphs keep pointing into theirs)
   std::vector<char*> chunks;
@@ -1257,6 +1459,8 @@ struct BatchPlan {
       if (x) cudaStreamDestroy(x);
     if (ev_in) cudaEventDestroy(ev_in);
     if (ev_out) cudaEventDestroy(ev_out);
+    for (cudaEvent_t e : {ev_fork, ev_join[0], ev_join[1]})
+      if (e) cudaEventDestroy(e);
   }
 };
 
@@ -1324,6 +1528,7 @@ int ensure_stream_ws(bd_state* s) {
 // one batched solve: elliptic (v -> u, all nodes) or parabolic (the
 // condensed systems of the tissue rows)
 struct BatchSolveArgs {
+  std::vector<bd_state*> mem;      // handle of each system
   bool elliptic;
   double alpha, c1, c2;            // parabolic: shift and right-hand-side factors
   bool node_terms;
@@ -1331,9 +1536,61 @@ struct BatchSolveArgs {
   std::vector<double*> x;
 };
 
+// the cluster-resident systems of a batched solve: one launch per kernel shape
+// (a cluster per system), launches of different shapes side by side; returns
+// the other systems' indices in rest
+int batch_solve_resident(BatchPlan& B, const BatchSolveArgs& q, cudaStream_t st, std::vector<int>* rest) {
+  bd_state* s0 = B.m[0];
+  const bool mixed = s0->precision == BD_MIXED;
+  struct Group {
+    ResShape shape;
+    bool amg;
+    size_t smem;
+    std::vector<ResLaunch> tab;
+  };
+  std::vector<Group> groups;
+  for (size_t r = 0; r < q.mem.size(); ++r) {
+    bd_state* s = q.mem[r];
+    if (!s->res_on) {
+      rest->push_back(int(r));
+      continue;
+    }
+    ResLaunch A = q.elliptic ? res_elliptic(s, q.va[r], q.x[r])
+                             : res_parabolic(s, q.alpha, q.c1, q.va[r], q.c2, q.vb[r], q.x[r], q.node_terms, true);
+    if (!A.valA || !A.valT) return fail(s0, BD_ERR_OOM, "device allocation failed");
+    A.gate = nullptr;
+    const bool amg = A.use_amg != 0;
+    Group* g = nullptr;
+    for (Group& x : groups)
+      if (x.amg == amg && x.shape.C == s->res.C && x.shape.block == s->res.block && x.shape.rpt == s->res.rpt) g = &x;
+    if (!g) {
+      groups.push_back(Group{s->res, amg, 0, {}});
+      g = &groups.back();
+    }
+    g->smem = std::max(g->smem, res_smem_bytes(s->res, mixed, amg));
+    g->tab.push_back(A);
+  }
+  if (groups.size() > 1) BCK(cudaEventRecord(B.ev_fork, st));
+  for (size_t k = 0; k < groups.size(); ++k) {
+    const Group& g = groups[k];
+    const cudaStream_t to = k == 0 ? st : B.side[(k - 1) % 2];
+    if (k > 0 && k <= 2) BCK(cudaStreamWaitEvent(to, B.ev_fork, 0));
+    B.enq += 1;
+    BCK(res_solve(g.shape, mixed, g.amg, nullptr, int(g.tab.size()), put(B, g.tab), g.smem, to));
+  }
+  for (size_t k = 0; k < 2 && k + 1 < groups.size(); ++k) {
+    BCK(cudaEventRecord(B.ev_join[k], B.side[k]));
+    BCK(cudaStreamWaitEvent(st, B.ev_join[k], 0));
+  }
+  return BD_OK;
+}
+
 int batch_solve(BatchPlan& B, const BatchSolveArgs& q, cudaStream_t st) {
   bd_state* s0 = B.m[0];
-  const int nseg = int(B.m.size());
+  std::vector<int> rest;
+  RUN(batch_solve_resident(B, q, st, &rest));
+  if (rest.empty()) return BD_OK;
+  const int nseg = int(rest.size());
   const bool mixed = s0->precision == BD_MIXED;
   std::vector<StreamLaunch> tab(nseg);
   std::vector<int> rows(nseg), post0(nseg), coarse(nseg);
@@ -1342,7 +1599,8 @@ int batch_solve(BatchPlan& B, const BatchSolveArgs& q, cudaStream_t st) {
   std::vector<AmgDev> hd(q.elliptic && !mixed ? nseg : 0);
   std::vector<std::vector<int>> lA(kMaxAmgLevels, std::vector<int>(nseg, 0)), lR = lA, lP = lA;
   for (int r = 0; r < nseg; ++r) {
-    bd_state* s = B.m[r];
+    const int sys = rest[r];
+    bd_state* s = q.mem[sys];
     const int n = int(q.elliptic ? s->N : s->NT);
     StreamLaunch A = stream_base(s, n);
     A.launch_acc = nullptr;
@@ -1353,7 +1611,7 @@ int batch_solve(BatchPlan& B, const BatchSolveArgs& q, cudaStream_t st) {
       A.valT = mixed ? static_cast<const void*>(s->fAie) : static_cast<const void*>(s->Aie);
       set_vec4(s, A, s->fAie4);
       A.val1 = s->Ai;
-      A.va = q.va[r];
+      A.va = q.va[sys];
       A.c1 = -1.0;
       A.project = 1;
       A.warm = 1;
@@ -1402,11 +1660,11 @@ int batch_solve(BatchPlan& B, const BatchSolveArgs& q, cudaStream_t st) {
       A.dextra = q.node_terms ? s->dgs : nullptr;
       A.rl = q.node_terms ? s->rl : nullptr;
       A.val1 = s->Ai;
-      A.va = q.va[r];
+      A.va = q.va[sys];
       A.c1 = q.c1;
-      if (!q.vb.empty() && q.vb[r]) {
+      if (q.vb[sys]) {
         A.val2 = s->Mv;
-        A.vb = q.vb[r];
+        A.vb = q.vb[sys];
         A.c2 = q.c2;
       }
       A.project = 0;
@@ -1422,7 +1680,7 @@ int batch_solve(BatchPlan& B, const BatchSolveArgs& q, cudaStream_t st) {
       A.outer_acc = s->d_stats + 5;
       post0[r] = 1;
     }
-    A.x = q.x[r];
+    A.x = q.x[sys];
     rows[r] = A.grid;
     tab[r] = A;
   }
@@ -1501,9 +1759,25 @@ int enqueue_batch_step(BatchPlan& B, double dt, int M, int K) {
     BatchSolveArgs q{};
     q.elliptic = true;
     for (bd_state* s : B.m) {
+      q.mem.push_back(s);
       q.va.push_back(s->NT < s->N ? s->vfull : vof(s));
       q.x.push_back(uof(s));
     }
+    return batch_solve(B, q, st);
+  };
+  // both elliptic constraints of a later sweep (M = 3) at once, for batches
+  // whose solves are all cluster-resident and need no zero-padded potentials
+  bool pairs = M == 3;
+  for (bd_state* s : B.m) pairs = pairs && s->res_on && s->NT == s->N;
+  auto elliptic_pairs = [&]() -> int {
+    BatchSolveArgs q{};
+    q.elliptic = true;
+    for (int m = 1; m <= 2; ++m)
+      for (bd_state* s : B.m) {
+        q.mem.push_back(s);
+        q.va.push_back(s->Xc[m]);
+        q.x.push_back(s->u[m]);
+      }
     return batch_solve(B, q, st);
   };
   auto parabolic_all = [&](double alpha, double c1, double c2, bool with_b, int m, int g) -> int {
@@ -1514,6 +1788,7 @@ int enqueue_batch_step(BatchPlan& B, double dt, int M, int K) {
     q.c2 = c2;
     q.node_terms = true;
     for (bd_state* s : B.m) {
+      q.mem.push_back(s);
       q.va.push_back(s->avec);
       q.vb.push_back(with_b ? s->bvec : nullptr);
       q.x.push_back(s->kinc[m][g]);
@@ -1540,8 +1815,10 @@ int enqueue_batch_step(BatchPlan& B, double dt, int M, int K) {
         B.enq += 2;
         BCK(launch_extrap_batch(put(B, t), blk_vec_u, nseg, nb_vec_u, st));
       }
-      for (int m = 1; m < M; ++m)
-        RUN(elliptic_all([m](bd_state* s) { return s->Xc[m]; }, [m](bd_state* s) { return s->u[m]; }));
+      if (pairs) RUN(elliptic_pairs());
+      else
+        for (int m = 1; m < M; ++m)
+          RUN(elliptic_all([m](bd_state* s) { return s->Xc[m]; }, [m](bd_state* s) { return s->u[m]; }));
     }
     // ROS2 predictor (the launch arguments of enqueue_step)
     for (int m = 0; m + 1 < M; ++m) {
@@ -2063,14 +2340,15 @@ int bd_create(const bd_mesh_t* mesh, const bd_cond_t* cond, bd_ionic_t model, co
     delete s;
     return fail(nullptr, BD_ERR_CUDA, "FP32 operator copy failed");
   }
-  if (s->opts.elliptic_precond == 1) {
-    rc = setup_amg(s, H);
-    if (rc != BD_OK) {
-      std::string m = s->err;
-      release(s);
-      delete s;
-      return fail(nullptr, rc, "%s", m.c_str());
-    }
+  AmgHost AH;
+  bool built = false;
+  rc = setup_resident(s, H, h_sptr, h_sw, &AH, &built);
+  if (rc == BD_OK && s->opts.elliptic_precond == 1) rc = setup_amg(s, H, AH, built);
+  if (rc != BD_OK) {
+    std::string m = s->err;
+    release(s);
+    delete s;
+    return fail(nullptr, rc, "%s", m.c_str());
   }
   s->host = std::move(H);
   // resting initial state
@@ -2187,6 +2465,9 @@ int bd_batch_step(bd_state_t* const* states, int n, double dt, int M, int K) {
         return fail(s0, BD_ERR_CUDA, "batch stream creation failed");
     if (cudaEventCreateWithFlags(&P->ev_in, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&P->ev_out, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&P->ev_join[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&P->ev_join[1], cudaEventDisableTiming) != cudaSuccess ||
         cudaMalloc(&P->ctl, sizeof(BatchCtl)) != cudaSuccess || cudaMemset(P->ctl, 0, sizeof(BatchCtl)) != cudaSuccess)
       return fail(s0, BD_ERR_CUDA, "batch set-up failed");
     g_batches.push_back(std::move(P));
@@ -2207,7 +2488,7 @@ int bd_batch_step(bd_state_t* const* states, int n, double dt, int M, int K) {
   }
   B->last_use = ++g_batch_clock;
   for (bd_state* h : B->m) {
-    RUN(ensure_stream_ws(h));
+    if (!h->res_on) RUN(ensure_stream_ws(h));
     RUN(prepare_step(h, dt, M));
   }
   // the members' queued work precedes the batch on the first handle's stream
