@@ -26,12 +26,20 @@
 //           computed sparsity lies inside ROWMASK[r].
 #pragma once
 #include <cmath>
+#include "fixexp.h"
 #include "sd.cuh"
 
 namespace bd {
 
 // ---- precision-dispatched elementary functions ----------------------------
-BD_HD double fexp(double x) { return exp(x); }
+// (host evaluations serve the resting state only)
+BD_HD double fexp(double x) {
+#ifdef __CUDA_ARCH__
+  return exp_fixed(x);
+#else
+  return exp(x);
+#endif
+}
 BD_HD double flog(double x) { return log(x); }
 BD_HD double fsqrt(double x) { return sqrt(x); }
 BD_HD float fexp(float x) {
