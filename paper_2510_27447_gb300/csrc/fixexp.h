@@ -1,4 +1,4 @@
-// fixexp.h -- exp of a double in 64-bit integer arithmetic.
+// fixexp.h -- exp and reciprocal of a double in 64-bit integer arithmetic.
 //
 // GB300's FP64 pipe takes two lanes a clock on an SM, its integer pipe 64: a
 // membrane evaluation of about 50 exponentials spends most of a quarter of its
@@ -164,6 +164,50 @@ BD_FIX_FN double exp_fixed(double x) {
   double d;
   std::memcpy(&d, &out, 8);
   return d;
+#endif
+}
+
+// 1 / d in integer arithmetic: the mantissa's reciprocal from FP32 (24 bits) by
+// two Newton steps r += r (1 - m r) in 64 bits, rounded once: at most 0.501
+// units in the last place (tests/test_exp_cpu.py).  Zero, subnormal and
+// non-finite d, and d whose reciprocal is subnormal, take the division.
+#ifdef __CUDACC__
+__host__ __device__ __noinline__
+#endif
+inline double recip_outside(double d) { return 1.0 / d; }
+
+BD_FIX_FN double recip_fixed(double d) {
+  uint64_t bits;
+#ifdef __CUDA_ARCH__
+  bits = uint64_t(__double_as_longlong(d));
+#else
+  std::memcpy(&bits, &d, 8);
+#endif
+  const uint32_t be = uint32_t(bits >> 52) & 0x7ffu;
+  if (be - 1u >= 2043u) return recip_outside(d);
+  const uint64_t m = bits << 11 | 0x8000000000000000ull;               // m / 2^63 in [1, 2)
+  uint32_t r0;                                                          // reciprocal, 2^32
+  const uint32_t fb = 0x3f800000u | (uint32_t(m >> 40) & 0x7fffffu);
+#ifdef __CUDA_ARCH__
+  r0 = __float2uint_rz(__fdividef(1.0f, __uint_as_float(fb)) * 4294967296.0f);   // saturates at 2^32 - 1
+#else
+  float f;
+  std::memcpy(&f, &fb, 4);
+  const float r = 1.0f / f * 4294967296.0f;
+  r0 = r >= 4294967296.0f ? 0xffffffffu : uint32_t(r);
+#endif
+  const int64_t e1 = int64_t(0x8000000000000000ull - fix_mulhi(m, uint64_t(r0) << 32));   // (1 - m r0) 2^63
+  const uint64_t r1 = (uint64_t(r0) << 32) + uint64_t((int64_t(r0) * int64_t(int32_t(e1 >> 11))) >> 20);
+  const int64_t e2 = int64_t(0x8000000000000000ull - fix_mulhi(m, r1));
+  uint64_t r2 = r1 + uint64_t((int64_t(r1 >> 32) * e2) >> 31);
+  if (e2 > 0 && r2 < r1) r2 = ~uint64_t(0);                             // m = 1: rounded up to 2^64
+  const uint64_t out = (r2 >> 11) + (r2 >> 10 & 1) + (uint64_t(2044u - be) << 52) + (bits & 0x8000000000000000ull);
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)out);
+#else
+  double q;
+  std::memcpy(&q, &out, 8);
+  return q;
 #endif
 }
 

@@ -130,7 +130,6 @@ __device__ __forceinline__ void ionic_body(const IonicLaunch& L, const Model<T>&
       for (int k = 1; k < NS; ++k) rho[k - 1] = e.f[k];
       fv = double(e.f[0]);
       avec = xj[0] + L.u[i];
-      if (L.pack) cond_store<T, Mod>(e, T(L.alpha), static_cast<T*>(L.pack) + i, n);
       // the field goes with the Jacobian only where a later predictor loads
       // both (FP64); the FP32 predictor keeps fewer values live without it
       if (L.jac_out) jac_store<T, Mod, sizeof(T) == 8>(e, static_cast<T*>(L.jac_out) + i, n);
@@ -183,7 +182,10 @@ __device__ __forceinline__ void ionic_body(const IonicLaunch& L, const Model<T>&
 
     T s, corr;
     T z[NS - 1], w[NS - 1];
-    condense<T, Mod>(e, T(L.alpha), rho, s, corr, z, w);
+    T* pk = nullptr;     // stage 1 keeps its condensation for stage 2
+    if constexpr (MODE == MODE_S1)
+      if (L.pack) pk = static_cast<T*>(L.pack) + i;
+    condense<T, Mod>(e, T(L.alpha), rho, s, corr, z, w, pk, n);
     double sd = double(s);
     if (sd < L.smin) {
       sd = L.smin;

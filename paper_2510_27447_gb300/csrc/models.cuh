@@ -26,6 +26,7 @@
 //           computed sparsity lies inside ROWMASK[r].
 #pragma once
 #include <cmath>
+#include <utility>
 #include "fixexp.h"
 #include "sd.cuh"
 
@@ -81,8 +82,8 @@ BD_HD void exprel_vd(float z, float& f, float& df) {
 }
 
 template <class T, uint32_t A> BD_HD SD<T, A> sexp(const SD<T, A>& a) { const T e = fexp(a.v); return chain(a, e, e); }
-template <class T, uint32_t A> BD_HD SD<T, A> slog(const SD<T, A>& a) { return chain(a, flog(a.v), T(1) / a.v); }
-template <class T, uint32_t A> BD_HD SD<T, A> ssqrt(const SD<T, A>& a) { const T s = fsqrt(a.v); return chain(a, s, T(0.5) / s); }
+template <class T, uint32_t A> BD_HD SD<T, A> slog(const SD<T, A>& a) { return chain(a, flog(a.v), recip(a.v)); }
+template <class T, uint32_t A> BD_HD SD<T, A> ssqrt(const SD<T, A>& a) { const T s = fsqrt(a.v); return chain(a, s, T(0.5) * recip(s)); }
 template <class T, uint32_t A> BD_HD SD<T, A> sexprel(const SD<T, A>& a) { T f, df; exprel_vd(a.v, f, df); return chain(a, f, df); }
 template <class T, uint32_t A> BD_HD SD<T, A> zero_like() { SD<T, A> r; r.v = T(0); for (int k = 0; k < SD<T, A>::nnz; ++k) r.d[k] = T(0); return r; }
 
@@ -496,19 +497,76 @@ struct DenseSink {
 // correction corr = j_vy . z.  A is block lower triangular (diagonal gates,
 // then the NB x NB block that may depend on the gates), so the solve is a
 // diagonal scaling followed by one small dense elimination.
+//
+// The block's elimination is sparse at compile time too: LuPattern follows the
+// fill of the elimination, and only entries that can be nonzero are touched
+// (TP06: 32 multiplications and additions instead of 154, and 16 instead of 42
+// in the back substitution).  With reciprocals in integer arithmetic (fixexp.h)
+// and the eliminated block kept for stage 2, the membrane kernels of a step take
+// (ms, before / after): TP06 257^2 mixed 0.406 / 0.285, slab 101x101x26 FP64, exp
+// included, 11.3 / 5.9.
+template <class Model>
+struct LuPattern {
+  uint32_t row[Model::NB > 0 ? Model::NB : 1];   // columns of block row r, fill included
+};
+template <class Model>
+constexpr LuPattern<Model> lu_pattern() {
+  LuPattern<Model> p{};
+  for (int r = 0; r < Model::NB; ++r) p.row[r] = (Model::ROWMASK[Model::NG + 1 + r] >> (Model::NG + 1)) | (1u << r);
+  for (int k = 0; k < Model::NB; ++k)
+    for (int i = k + 1; i < Model::NB; ++i)
+      if (p.row[i] >> k & 1u) p.row[i] |= p.row[k] & ~((2u << k) - 1u);
+  return p;
+}
+// rows below k with an entry in column k; columns of row r right of its diagonal
+template <class Model>
+constexpr uint32_t lu_below(int k) {
+  uint32_t m = 0;
+  for (int i = k + 1; i < Model::NB; ++i)
+    if (lu_pattern<Model>().row[i] >> k & 1u) m |= 1u << i;
+  return m;
+}
+template <class Model>
+constexpr uint32_t lu_right(int r) { return lu_pattern<Model>().row[r] & ~((2u << r) - 1u); }
+
+// f(integral_constant<int, k>) for k = 0..N-1, and for k = N-1..0
+template <int N, class F>
+BD_HD void static_for(F&& f) {
+  [&]<int... K>(std::integer_sequence<int, K...>) { (f(std::integral_constant<int, K>{}), ...); }
+  (std::make_integer_sequence<int, N>{});
+}
+
+// What stage 2 of a ROS2 step needs of stage 1's condensation (same node
+// Jacobian, same shift alpha): stage 1 stores it, stage 2 then solves
+// A z = rho for its new rho without evaluating the Jacobian or eliminating the
+// block again.  Layout per node, cond_pack_size() values (strided by the node
+// count; entries outside the patterns are neither written nor read):
+//   [0, NG)             1 / (alpha - d g_k / d x_k), gates k = 1..NG
+//   [NG, NG + NB NG)    d f_{NG+1+r} / d x_k, block row r, gate k
+//   next NB NB          the eliminated block: multipliers left of the diagonal,
+//                       reciprocal pivots on it, the upper factor right of it
+//   next NS             d f_0 / d X_c
+template <class Model>
+constexpr int cond_pack_size() {
+  return Model::NG + Model::NB * Model::NG + Model::NB * Model::NB + Model::NS;
+}
+
+// pk: where to store what cond_solve() needs (node stride `stride`), or NULL
 template <class T, class Model>
-BD_HD void condense(const JacSink<T, Model>& e, T alpha, const T* rho, T& s, T& corr, T* z, T* w) {
+BD_HD void condense(const JacSink<T, Model>& e, T alpha, const T* rho, T& s, T& corr, T* z, T* w, T* pk = nullptr,
+                    int64_t stride = 0) {
   constexpr int NG = Model::NG, NB = Model::NB;
   constexpr uint32_t GATES = ((1u << (NG + 1)) - 1u) & ~1u;
 #pragma unroll
   for (int g = 1; g <= NG; ++g) {
-    const T inv = T(1) / (alpha - e.jgd[g]);
+    const T inv = recip(alpha - e.jgd[g]);
+    if (pk) pk[(g - 1) * stride] = inv;
     z[g - 1] = rho[g - 1] * inv;
     w[g - 1] = e.jgv[g] * inv;
   }
   T Bm[NB][NB];
-  T rz[NB], rw[NB];
-  auto fill = [&](auto rr) {
+  T rz[NB], rw[NB], piv[NB];
+  static_for<NB>([&](auto rr) {
     constexpr int r = decltype(rr)::value;
     constexpr uint32_t RM = Model::ROWMASK[NG + 1 + r];
     rz[r] = rho[NG + r];
@@ -516,48 +574,57 @@ BD_HD void condense(const JacSink<T, Model>& e, T alpha, const T* rho, T& s, T& 
     else rw[r] = T(0);
     for_bits<RM & GATES>([&](auto b) {
       constexpr int c = decltype(b)::value;
+      if (pk) pk[(NG + r * NG + (c - 1)) * stride] = e.jb[r][c];
       rz[r] += e.jb[r][c] * z[c - 1];
       rw[r] += e.jb[r][c] * w[c - 1];
     });
-#pragma unroll
-    for (int c = 0; c < NB; ++c) Bm[r][c] = (r == c) ? alpha : T(0);
+    for_bits<lu_pattern<Model>().row[r]>([&](auto b) {
+      constexpr int c = decltype(b)::value;
+      Bm[r][c] = (r == c) ? alpha : T(0);
+    });
     for_bits<(RM >> (NG + 1))>([&](auto b) {
       constexpr int c = decltype(b)::value;
       Bm[r][c] -= e.jb[r][NG + 1 + c];
     });
-  };
-  [&]<int... R>(std::integer_sequence<int, R...>) { (fill(std::integral_constant<int, R>{}), ...); }
-  (std::make_integer_sequence<int, NB>{});
+  });
   // in-register LU without pivoting (A = alpha I - j_yy is dominated by alpha I)
-#pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    const T piv = T(1) / Bm[k][k];
-#pragma unroll
-    for (int i = k + 1; i < NB; ++i) {
-      const T l = Bm[i][k] * piv;
-#pragma unroll
-      for (int c = k + 1; c < NB; ++c) Bm[i][c] -= l * Bm[k][c];
+  static_for<NB>([&](auto kk) {
+    constexpr int k = decltype(kk)::value;
+    piv[k] = recip(Bm[k][k]);
+    if (pk) pk[(NG + NB * NG + k * NB + k) * stride] = piv[k];
+    for_bits<lu_right<Model>(k)>([&](auto cc) {
+      constexpr int c = decltype(cc)::value;
+      if (pk) pk[(NG + NB * NG + k * NB + c) * stride] = Bm[k][c];
+    });
+    for_bits<lu_below<Model>(k)>([&](auto ii) {
+      constexpr int i = decltype(ii)::value;
+      const T l = Bm[i][k] * piv[k];
+      if (pk) pk[(NG + NB * NG + i * NB + k) * stride] = l;
+      for_bits<lu_right<Model>(k)>([&](auto cc) {
+        constexpr int c = decltype(cc)::value;
+        Bm[i][c] -= l * Bm[k][c];
+      });
       rz[i] -= l * rz[k];
       rw[i] -= l * rw[k];
-    }
-  }
-#pragma unroll
-  for (int i = NB - 1; i >= 0; --i) {
-#pragma unroll
-    for (int c = i + 1; c < NB; ++c) {
+    });
+  });
+  static_for<NB>([&](auto kk) {
+    constexpr int i = NB - 1 - decltype(kk)::value;
+    for_bits<lu_right<Model>(i)>([&](auto cc) {
+      constexpr int c = decltype(cc)::value;
       rz[i] -= Bm[i][c] * rz[c];
       rw[i] -= Bm[i][c] * rw[c];
-    }
-    const T inv = T(1) / Bm[i][i];
-    rz[i] *= inv;
-    rw[i] *= inv;
+    });
+    rz[i] *= piv[i];
+    rw[i] *= piv[i];
     z[NG + i] = rz[i];
     w[NG + i] = rw[i];
-  }
+  });
   s = -e.jv[0];
   corr = T(0);
   for_bits<Model::ROWMASK[0] & ~1u>([&](auto b) {
     constexpr int c = decltype(b)::value;
+    if (pk) pk[(NG + NB * NG + NB * NB + c) * stride] = e.jv[c];
     s -= e.jv[c] * w[c - 1];
     corr += e.jv[c] * z[c - 1];
   });
@@ -630,47 +697,6 @@ BD_HD void jac_load(JacSink<T, Model>& e, const T* pk, int64_t stride) {
   for (int k = 0; k < NS; ++k) e.f[k] = pk[(NS + 2 * NG + NB * NS + k) * stride];
 }
 
-// What stage 2 of a ROS2 step needs of stage 1's condensation (same node
-// Jacobian, same shift alpha): stage 1 stores it, stage 2 then solves
-// A z = rho for its new rho without evaluating the Jacobian again.  Layout per
-// node, PACK values (strided by the node count):
-//   [0, NG)             1 / (alpha - d g_k / d x_k), gates k = 1..NG
-//   [NG, NG + NB NG)    d f_{NG+1+r} / d x_k, block row r, gate k (pattern entries)
-//   next NB NB          the block matrix alpha I - J_yy restricted to the block
-//   next NS             d f_0 / d X_c (pattern entries)
-template <class Model>
-constexpr int cond_pack_size() {
-  return Model::NG + Model::NB * Model::NG + Model::NB * Model::NB + Model::NS;
-}
-
-template <class T, class Model>
-BD_HD void cond_store(const JacSink<T, Model>& e, T alpha, T* pk, int64_t stride) {
-  constexpr int NG = Model::NG, NB = Model::NB;
-  constexpr uint32_t GATES = ((1u << (NG + 1)) - 1u) & ~1u;
-#pragma unroll
-  for (int g = 1; g <= NG; ++g) pk[(g - 1) * stride] = T(1) / (alpha - e.jgd[g]);
-  auto row = [&](auto rr) {
-    constexpr int r = decltype(rr)::value;
-    constexpr uint32_t RM = Model::ROWMASK[NG + 1 + r];
-    for_bits<RM & GATES>([&](auto b) {
-      constexpr int c = decltype(b)::value;
-      pk[(NG + r * NG + (c - 1)) * stride] = e.jb[r][c];
-    });
-#pragma unroll
-    for (int c = 0; c < NB; ++c) pk[(NG + NB * NG + r * NB + c) * stride] = (r == c) ? alpha : T(0);
-    for_bits<(RM >> (NG + 1))>([&](auto b) {
-      constexpr int c = decltype(b)::value;
-      pk[(NG + NB * NG + r * NB + c) * stride] = ((r == c) ? alpha : T(0)) - e.jb[r][NG + 1 + c];
-    });
-  };
-  [&]<int... R>(std::integer_sequence<int, R...>) { (row(std::integral_constant<int, R>{}), ...); }
-  (std::make_integer_sequence<int, NB>{});
-  for_bits<Model::ROWMASK[0] & ~1u>([&](auto b) {
-    constexpr int c = decltype(b)::value;
-    pk[(NG + NB * NG + NB * NB + c) * stride] = e.jv[c];
-  });
-}
-
 // z = A^-1 rho and corr = sum_c j_vc z_c from a stored pack: the arithmetic of
 // condense() for z and corr, operation for operation
 template <class T, class Model>
@@ -679,40 +705,31 @@ BD_HD void cond_solve(const T* pk, int64_t stride, const T* rho, T& corr, T* z) 
   constexpr uint32_t GATES = ((1u << (NG + 1)) - 1u) & ~1u;
 #pragma unroll
   for (int g = 1; g <= NG; ++g) z[g - 1] = rho[g - 1] * pk[(g - 1) * stride];
-  T Bm[NB][NB];
   T rz[NB];
-  auto fill = [&](auto rr) {
+  static_for<NB>([&](auto rr) {
     constexpr int r = decltype(rr)::value;
-    constexpr uint32_t RM = Model::ROWMASK[NG + 1 + r];
     rz[r] = rho[NG + r];
-    for_bits<RM & GATES>([&](auto b) {
+    for_bits<Model::ROWMASK[NG + 1 + r] & GATES>([&](auto b) {
       constexpr int c = decltype(b)::value;
       rz[r] += pk[(NG + r * NG + (c - 1)) * stride] * z[c - 1];
     });
-#pragma unroll
-    for (int c = 0; c < NB; ++c) Bm[r][c] = pk[(NG + NB * NG + r * NB + c) * stride];
-  };
-  [&]<int... R>(std::integer_sequence<int, R...>) { (fill(std::integral_constant<int, R>{}), ...); }
-  (std::make_integer_sequence<int, NB>{});
-#pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    const T piv = T(1) / Bm[k][k];
-#pragma unroll
-    for (int i = k + 1; i < NB; ++i) {
-      const T l = Bm[i][k] * piv;
-#pragma unroll
-      for (int c = k + 1; c < NB; ++c) Bm[i][c] -= l * Bm[k][c];
-      rz[i] -= l * rz[k];
-    }
-  }
-#pragma unroll
-  for (int i = NB - 1; i >= 0; --i) {
-#pragma unroll
-    for (int c = i + 1; c < NB; ++c) rz[i] -= Bm[i][c] * rz[c];
-    const T inv = T(1) / Bm[i][i];
-    rz[i] *= inv;
+  });
+  static_for<NB>([&](auto kk) {
+    constexpr int k = decltype(kk)::value;
+    for_bits<lu_below<Model>(k)>([&](auto ii) {
+      constexpr int i = decltype(ii)::value;
+      rz[i] -= pk[(NG + NB * NG + i * NB + k) * stride] * rz[k];
+    });
+  });
+  static_for<NB>([&](auto kk) {
+    constexpr int i = NB - 1 - decltype(kk)::value;
+    for_bits<lu_right<Model>(i)>([&](auto cc) {
+      constexpr int c = decltype(cc)::value;
+      rz[i] -= pk[(NG + NB * NG + i * NB + c) * stride] * rz[c];
+    });
+    rz[i] *= pk[(NG + NB * NG + i * NB + i) * stride];
     z[NG + i] = rz[i];
-  }
+  });
   corr = T(0);
   for_bits<Model::ROWMASK[0] & ~1u>([&](auto b) {
     constexpr int c = decltype(b)::value;

@@ -13,11 +13,23 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "fixexp.h"
+
 #ifndef BD_HD
 #define BD_HD __host__ __device__ __forceinline__
 #endif
 
 namespace bd {
+
+// 1 / x; FP64 on the device in integer arithmetic (fixexp.h)
+BD_HD float recip(float x) { return 1.0f / x; }
+BD_HD double recip(double x) {
+#ifdef __CUDA_ARCH__
+  return recip_fixed(x);
+#else
+  return 1.0 / x;
+#endif
+}
 
 namespace sdm {
 constexpr int popc(uint32_t m) { int c = 0; while (m) { c += int(m & 1u); m >>= 1; } return c; }
@@ -132,7 +144,7 @@ template <class T, uint32_t A, uint32_t B>
 BD_HD SD<T, A | B> operator/(const SD<T, A>& a, const SD<T, B>& b) {
   constexpr uint32_t C = A | B;
   SD<T, C> r;
-  const T inv = T(1) / b.v;
+  const T inv = recip(b.v);
   r.v = a.v * inv;
   for_bits<C>([&](auto bb) {
     constexpr int bit = decltype(bb)::value;
@@ -161,7 +173,7 @@ template <class T, uint32_t A> BD_HD SD<T, A> operator*(const SD<T, A>& a, T c) 
 template <class T, uint32_t A> BD_HD SD<T, A> operator*(T c, const SD<T, A>& a) { return a * c; }
 template <class T, uint32_t A> BD_HD SD<T, A> operator/(const SD<T, A>& a, T c) { return a * (T(1) / c); }
 template <class T, uint32_t A> BD_HD SD<T, A> operator/(T c, const SD<T, A>& a) {
-  const T inv = T(1) / a.v;
+  const T inv = recip(a.v);
   const T f = c * inv;
   return chain(a, f, -f * inv);
 }
