@@ -414,7 +414,7 @@ cudaError_t launch_sell_v4(int64_t n_slices, const int64_t* sptr, const int* sw,
 // kernels set, so a solve needs no host round trip.
 struct StreamScal {               // device scalars of one streaming solve
   double mean_b, bb, tol2;        // right-hand side mean (projected systems), |b|^2, tol^2 |b|^2
-  double rr64, scale, tgt;        // outer residual, its norm, inner target (relative, squared)
+  double rr64, scale, inv_scale, tgt;   // outer residual, its norm and 1 / norm, inner target (relative, squared)
   double rr_new, rho, alpha, beta, shift;
   int outer, it, fail, stop, inner_ran, skip, first, more;   // more: wants another outer pass
   long long inner_total, outer_total;

@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kSB) st_rhs_kernel(const __grid_constant__ S s
     if (!a.use_amg) {
       double d = a.valA[a.diagpos[i]];
       if (a.dextra) d += a.dextra[i];
-      invd[i] = T(1.0 / d);
+      invd[i] = T(1) / T(d);   // FP32: no FP64 division per row
     }
     if (!a.warm) a.x[i] = 0.0;
     acc[0] += b;
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kSB) st_inner_init_kernel(const __grid_constan
   const T* invd0 = static_cast<const T*>(a.h0_invd);
   T* x0 = static_cast<T*>(a.h0_x);
   const T omega0 = T(a.h0_omega);
-  const double inv_scale = 1.0 / c.scale;
+  const double inv_scale = c.inv_scale;
   T acc[2] = {T(0), T(0)};
   for (int i = gt; i < a.n; i += gs) {
     const T ri = T(a.r64[i] * inv_scale);

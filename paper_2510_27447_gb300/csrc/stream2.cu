@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kSB) st2_inner_init_kernel(const __grid_consta
   T acc[2] = {T(0), T(0)};
   by_mask(on0, on1, [&](auto m) {
     MASK_OF(m);
-    const double inv_scale[2] = {1.0 / P.a[0].sc->scale, 1.0 / P.a[1].sc->scale};
+    const double inv_scale[2] = {P.a[0].sc->inv_scale, P.a[1].sc->inv_scale};
     for (int i = gt; i < a.n; i += gs) {
       const T w = omega0 * invd0[i];
 #pragma unroll

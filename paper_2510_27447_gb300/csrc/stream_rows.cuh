@@ -349,6 +349,7 @@ __device__ __forceinline__ bool outer_decide(const StreamLaunch& a, double rr) {
     return false;
   }
   c.scale = sqrt(rr);
+  c.inv_scale = 1.0 / c.scale;   // here once: per thread of the grid it occupies the FP64 pipe for 7 us
   // inner target relative to |r|^2: the FP32 solves follow the persistent
   // mixed kernel; a single FP64 solve stops at |r| <= tol |b|, as the
   // persistent FP64 kernel does
