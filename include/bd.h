@@ -147,7 +147,12 @@ typedef struct {
                             Streaming solves chain full-occupancy kernels whose CG loops run on
                             the device as CUDA graph conditional nodes; persistent solves are
                             one cooperative kernel each (bd_stats_t.streaming reports the form
-                            in use) */
+                            in use).  With 0 the form is chosen per kind of solve: a mixed
+                            streaming handle's parabolic solves are persistent below 7M entries, a
+                            persistent handle's elliptic solves run as kernel chains inside its
+                            captured steps (use_graph) where those are faster: 3-D meshes,
+                            FP64 sheets of more than 77,824 nodes, mixed-precision sheets of
+                            more than 1M entries */
   int vec4;              /* 0 (default): mixed-precision streaming solves also keep the FP32
                             elliptic and parabolic operators, and every FP32 AMG level operator
                             stored as SELL-32 with at least 2^17 rows, in the SELL-32/4 layout
@@ -158,7 +163,8 @@ typedef struct {
                             give the same sums in the same order */
   int csr_lanes;         /* streaming solves, AMG levels stored as CSR: threads per row.  0
                             (default): a quarter of the level's mean row length rounded up to a
-                            power of two in [4, 32], or 256 (a block per row) for rows of 256
+                            power of two in [4, 32] (FP64, rows of more than 16: 8, or 16 or 32
+                            where there are few rows), or 256 (a block per row) for rows of 256
                             entries and more on average; 4, 8, 16, 32 or 256 force that width on
                             every CSR level (tuning and testing); BD_ERR_ARG otherwise */
   int wide_sell;         /* streaming handles, AMG levels with rows longer than 32 entries: 0
@@ -199,7 +205,7 @@ typedef struct {
                               entries) */
   int64_t amg_levels;      /* smoothed AMG levels of the elliptic preconditioner (0: Jacobi) */
   int64_t amg_coarse_rows; /* rows of the dense coarsest AMG level (0: Jacobi) */
-  int64_t streaming;       /* 1: the solves run as streaming kernel chains (bd_opts_t.streaming) */
+  int64_t streaming;       /* 1: a streaming handle, 0: a persistent one (bd_opts_t.streaming) */
 } bd_stats_t;
 
 /* Per-kind device time of profiled steps (bd_profile_steps). */

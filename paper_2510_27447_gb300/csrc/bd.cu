@@ -59,6 +59,40 @@ constexpr int64_t kNoAllocWords = 5 * kNoAllocRows + 4 * kNoAllocBlocks + 4;
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocWords];
 }  // namespace
 
+// Which elliptic solves of a persistent handle run as streaming kernel chains
+// (inside the steps the library captures: loops on the device need a graph):
+// the single ones and the two-system ones.  The persistent AMG kernels hold 16
+// or 32 warps an SM through every phase and, in FP64, a warp per CSR row and
+// one system at a time; the chain's kernels run at their own occupancy.
+// Measured, elliptic ms of a step persistent / chain, one solve (1 sweep) and
+// one + pair (2 sweeps):
+//   FP64   slab  31x31x8  1.37 / 0.76, 4.09 / 1.84;  101x101x26 4.38 / 3.37,
+//          12.7 / 8.30;  sheet 257^2 0.92 / 1.19, 2.68 / 2.86;  285^2 1.55 /
+//          1.45, 4.51 / 3.50;  513^2 2.45 / 1.95, 7.23 / 4.79
+//   mixed  slab 61x61x9   1.32 / 1.17, 2.98 / 2.48;  101x101x26 3.36 / 2.24,
+//          7.63 / 5.00;  sheet 257^2 0.69 / 1.04, 1.59 / 2.22;  401^2 1.37 /
+//          1.46, 3.38 / 3.15;  513^2 1.65 / 1.72, 3.97 / 3.57;  701^2 2.96 / 2.20
+// So: 3-D patterns always; 2-D ones in FP64 where the rows leave the
+// 512-thread build (77,824 = 152 x 512 rows), in mixed precision the pair from
+// 1M entries and the single solve from 2.5M.
+struct ChainRule {
+  bool one = false, two = false;
+};
+static ChainRule chain_rule(const bd_opts_t& o, int64_t N, int64_t nnz) {
+  ChainRule r;
+  if (o.streaming != 0 || !o.use_graph || o.cg_cluster != 0 || o.solver_tier != 0 || o.cg_block != 0 ||
+      o.cg_grid != 0 || o.elliptic_precond != 1 || N <= std::max(1500, o.amg_coarse_max) || nnz >= kStreamNnz)
+    return r;
+  const bool rows3d = nnz >= 10 * N;   // about 15 entries a row against 7
+  if (o.precision == BD_MIXED) {
+    r.one = rows3d || nnz >= 2500000;
+    r.two = rows3d || nnz >= 1000000;
+  } else {
+    r.one = r.two = rows3d || N > 152 * 512;
+  }
+  return r;
+}
+
 struct bd_state {
   int model = 0, ns = 0, dim = 0, precision = 0;
   int device = 0;                 // CUDA device current at bd_create (the handle's device)
@@ -156,6 +190,9 @@ struct bd_state {
   // streaming solver (operators that do not fit in L2): device scalars, block
   // partials, FP64-path workspaces and two streams that capture loop bodies
   bool streaming = false;
+  bool stream_par = false;        // ... and its parabolic solves take the form too (kStreamParNnz)
+  ChainRule chain{};              // persistent handles: elliptic solves that run as kernel chains inside captured steps
+  bool capturing = false;         // the library is capturing one of its steps
   StreamScal* d_sc = nullptr;     // two: a solve's (or a pair's first system's) and a pair's second system's
   double* spart = nullptr;
   double *sb64 = nullptr, *sr64 = nullptr;
@@ -520,6 +557,7 @@ StreamLaunch elliptic_launch(bd_state* s, const double* v, double* u, int k = 0)
   A.max_outer = mixed ? 12 : 1;
   A.inner_cap = s->opts.cg_cap_e;
   A.use_amg = s->use_amg ? 1 : 0;
+  A.strict = !s->streaming && !mixed;
   A.tol = s->opts.cg_tol_e;
   A.tol_inner = mixed ? double(BD_MIXED_TOL_INNER) : s->opts.cg_tol_e;
   A.iters_acc = s->d_stats + 0;
@@ -539,7 +577,7 @@ StreamLaunch elliptic_launch(bd_state* s, const double* v, double* u, int k = 0)
 }
 
 int elliptic(bd_state* s, const double* v, double* u) {
-  if (s->streaming) {
+  if (s->streaming || (s->capturing && s->chain.one)) {
     if (s->NT < s->N) {
       Timed t(s, BD_K_COMBINE);
       CK(launch_copy(s->NT, v, s->vfull, s->stream, s->opts.sweep_tol > 0 ? s->gate : nullptr));
@@ -614,13 +652,14 @@ int elliptic2(bd_state* s, const double* v1, double* u1, const double* v2, doubl
     return BD_OK;
   }
   // pairs: mixed AMG solves in both forms, FP64 AMG solves in the streaming form
-  const bool pair = s->use_amg && s->opts.pair_solve >= 0 && (mixed ? s->two_rhs : s->streaming && s->pair64);
+  const bool chain = s->streaming || (s->capturing && s->chain.two);
+  const bool pair = s->use_amg && s->opts.pair_solve >= 0 && (mixed ? s->two_rhs : chain && s->pair64);
   if (!pair) {
     const int r = elliptic(s, v1, u1);
     if (r != BD_OK) return r;
     return elliptic(s, v2, u2);
   }
-  if (s->streaming) {   // one chain for both systems (stream2.cu)
+  if (chain) {   // one chain for both systems (stream2.cu)
     if (s->NT < s->N) {
       if (!s->vfull || !s->vfull2) return fail(s, BD_ERR_ARG, "two-system solve without its full-length potentials");
       Timed t(s, BD_K_COMBINE, 2);
@@ -684,7 +723,7 @@ int parabolic(bd_state* s, double alpha, double c1, const double* va, double c2,
     CK(res_solve(s->res, s->precision == BD_MIXED, false, &A, 1, nullptr, 0, s->stream));
     return BD_OK;
   }
-  if (s->streaming) {
+  if (s->stream_par) {
     StreamLaunch A = stream_base(s, int(s->NT));   // tissue rows; their bath columns hold zeros
     const bool mixed = s->precision == BD_MIXED;
     A.valA = p_values(s, alpha);
@@ -925,7 +964,8 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH, bool built) {
     out->wmax = S.wmax;
     const bool csr = !S.rp.empty();
     out->rp = csr ? static_cast<const int64_t*>(upload(S.rp.data(), S.rp.size() * 8)) : nullptr;
-    out->lpr = csr ? (s->opts.csr_lanes > 0 ? s->opts.csr_lanes : csr_lanes(S.rp.back(), S.n)) : 0;
+    const bool f64 = s->precision == BD_FP64;
+    out->lpr = csr ? (s->opts.csr_lanes > 0 ? s->opts.csr_lanes : csr_lanes(S.rp.back(), S.n, f64)) : 0;
     out->sptr = csr ? nullptr : static_cast<const int64_t*>(upload(S.sptr.data(), S.sptr.size() * 8));
     out->sw = csr ? nullptr : static_cast<const int*>(upload(S.sw.data(), S.sw.size() * 4));
     out->col = static_cast<const int*>(upload(S.col.data(), S.col.size() * 4));
@@ -970,7 +1010,7 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH, bool built) {
   if (!M.cinv || !alloc_n(s, &M.bc, AH.nc) || !alloc_n(s, &M.xc, AH.nc) ||
       cudaStreamSynchronize(s->stream) != cudaSuccess)
     return fail(s, BD_ERR_OOM, "AMG upload failed");
-  if (s->precision == BD_FP64 && s->streaming && s->opts.pair_solve >= 0) {
+  if (s->precision == BD_FP64 && (s->streaming || s->chain.two) && s->opts.pair_solve >= 0) {
     // the same hierarchy with its own level vectors: the second system of the
     // streaming two-system solves (sweeps >= 2)
     AmgDev& G = s->amg2;
@@ -992,7 +1032,7 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH, bool built) {
       out->wmax = S.wmax;
       const bool csr = !S.rp.empty();
       out->rp = csr ? static_cast<const int64_t*>(upload(S.rp.data(), S.rp.size() * 8)) : nullptr;
-      out->lpr = csr ? (s->opts.csr_lanes > 0 ? s->opts.csr_lanes : csr_lanes(S.rp.back(), S.n)) : 0;
+      out->lpr = csr ? (s->opts.csr_lanes > 0 ? s->opts.csr_lanes : csr_lanes(S.rp.back(), S.n, false)) : 0;
       out->sptr = csr ? nullptr : static_cast<const int64_t*>(upload(S.sptr.data(), S.sptr.size() * 8));
       out->sw = csr ? nullptr : static_cast<const int*>(upload(S.sw.data(), S.sw.size() * 4));
       out->col = static_cast<const int*>(upload(S.col.data(), S.col.size() * 4));
@@ -1353,7 +1393,9 @@ int do_step(bd_state* s, double dt, int M, int K) {
     cudaGraph_t g = nullptr;
     s->enq_launches = 0;
     CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
+    s->capturing = true;
     const int r = enqueue_any(s, dt, M, K);
+    s->capturing = false;
     cudaError_t e = cudaStreamEndCapture(s->stream, &g);
     if (r != BD_OK) {
       if (g) cudaGraphDestroy(g);
@@ -1387,7 +1429,9 @@ int do_step(bd_state* s, double dt, int M, int K) {
       const int64_t ev0 = s->ionic_evals;
       s->enq_launches = 0;
       CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
+      s->capturing = true;
       const int r = enqueue_any(s, dt, M, K);
+      s->capturing = false;
       const int64_t nl = s->enq_launches;
       cudaError_t e = cudaStreamEndCapture(s->stream, &g);
       if (r != BD_OK) {
@@ -1404,7 +1448,18 @@ int do_step(bd_state* s, double dt, int M, int K) {
       s->ionic_evals = ev0;   // counted per replay below
     }
     s->launches_per_step = ge->launches;
-    CK(cudaGraphLaunch(ge->exec, s->stream));
+    // a caller's own capture takes the step as a child graph, which may not
+    // hold conditional nodes: a step with kernel chains goes in launch by
+    // launch instead, its elliptic solves in the persistent form
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (s->chain.one || s->chain.two) CK(cudaStreamIsCapturing(s->stream, &cs));
+    if (cs == cudaStreamCaptureStatusActive) {
+      const int64_t ev0 = s->ionic_evals;
+      RUN(enqueue_any(s, dt, M, K));
+      s->ionic_evals = ev0;
+    } else {
+      CK(cudaGraphLaunch(ge->exec, s->stream));
+    }
     s->launches += s->launches_per_step;
     s->ionic_evals += M == 0 ? 4 : int64_t(K) * (3 * (M - 1) + (s->opts.sdc_correction ? M : 0)) + 1;
   }
@@ -2211,9 +2266,11 @@ int bd_create(const bd_mesh_t* mesh, const bd_cond_t* cond, bd_ionic_t model, co
       return fail(nullptr, BD_ERR_ARG, "streaming = 2 (host-driven loops) needs sweep_tol = 0");
     }
     s->streaming = s->opts.cg_cluster == 0 && (so >= 1 || (so == 0 && nnz >= kStreamNnz));
+    s->stream_par = s->streaming && (so >= 1 || s->precision != BD_MIXED || nnz >= kStreamParNnz);
     if (so == 2) s->opts.use_graph = 0;   // host-driven loops cannot be captured
+    if (!res_wanted(s)) s->chain = chain_rule(s->opts, N, nnz);
   }
-  if (ok && s->streaming) {
+  if (ok && (s->streaming || s->chain.one || s->chain.two)) {
     stream_prepare();   // kernel occupancies, queried outside any capture
     ok = alloc_n(s, reinterpret_cast<char**>(&s->d_sc), int64_t(2 * sizeof(StreamScal))) &&
          alloc_n(s, &s->spart, int64_t(stream_grid_cap()) * 4);
@@ -2254,7 +2311,7 @@ int bd_create(const bd_mesh_t* mesh, const bd_cond_t* cond, bd_ionic_t model, co
       return fail(nullptr, BD_ERR_ARG, "pair_solve must be -1 or 0");
     }
   }
-  s->vec4 = s->streaming && s->precision == BD_MIXED && s->opts.vec4 >= 0;
+  s->vec4 = (s->streaming || s->chain.one || s->chain.two) && s->precision == BD_MIXED && s->opts.vec4 >= 0;
   std::vector<int64_t> h_sptr4;
   std::vector<int> e_col4;
   int64_t en4 = 0;
@@ -2764,12 +2821,13 @@ size_t bd_footprint_bytes(const bd_mesh_t* mesh, bd_ionic_t model, const bd_opts
   // FP32 operators (8 bytes an entry, widths padded to 4)
   const bool streaming =
       o.cg_cluster == 0 && (o.streaming >= 1 || (o.streaming == 0 && nnz >= double(kStreamNnz)));
-  if (streaming) {
+  const ChainRule chain = chain_rule(o, int64_t(N), int64_t(nnz));
+  if (streaming || chain.one || chain.two) {
     extra += N * 8 * 8;
     // FP64 two-system solves: second halves of seven workspaces and a second
     // set of AMG level vectors
     if (!mixed && amg && o.pair_solve >= 0) extra += N * 8 * 7 + N * 8 * 2.6;
-    if (mixed && o.vec4 >= 0) extra += (nnz * 5 + lev) * 8 * 1.15;
+    if (mixed && o.vec4 >= 0) extra += (nnz * (streaming ? 5 : 1) + lev) * 8 * 1.15;
   }
   return size_t(mat + st + packs + extra) + (size_t(1) << 20);
 }
@@ -2965,7 +3023,7 @@ int bd_profile_steps(bd_state_t* s, double dt, int M, int K, int n_steps, bd_pro
     out->coarse_bytes = cycles * s->amg_coarse_bytes[v];
     const double ncc = vb * double(s->amg.nc) * double(s->amg.nc);   // the dense coarse inverse
     out->vcycle_bytes -= (pairs + pairsc) * (s->amg_cycle_opbytes[v] - ncc);
-    if (s->streaming) out->coarse_bytes -= (pairs + pairsc) * ncc;   // read once for both systems
+    if (s->streaming || s->chain.two) out->coarse_bytes -= (pairs + pairsc) * ncc;   // read once for both systems
   }
   return read_status(s);
 }

@@ -26,8 +26,13 @@ constexpr int64_t kTier2Nnz = 12000000;
 // operators of at least kStreamNnz entries take the streaming solver form by
 // default (measured on GB300, mixed, ms per step persistent / streaming:
 // 513^2 sheet, 1.8M entries, 6.75 / 8.28; 3-D slab of 3.9M entries 11.7 /
-// 12.0; 1025^2 sheet, 7.3M, 19.3 / 17.9; 3-D slab of 10.6M 27.3 / 22.5)
+// 12.0; 1025^2 sheet, 7.3M, 19.3 / 17.9; 3-D slab of 10.6M 27.3 / 22.5).
+// The parabolic solves (Jacobi, two kernels an iteration) gain later than the
+// elliptic ones: in mixed precision from kStreamParNnz entries (their ms per
+// step persistent / streaming: slab of 5.1M entries 2.78 / 3.87; 1025^2 sheet,
+// 7.3M, 11.1 / 10.6; slab of 12M 7.28 / 5.70).
 constexpr int64_t kStreamNnz = 5000000;
+constexpr int64_t kStreamParNnz = 7000000;
 
 // device status word bits (one per bd_status_t failure kind)
 enum : int {
@@ -327,8 +332,19 @@ struct SellDevT {
 // and more on average (restrictions onto the coarsest level: few rows, long)
 // get a whole block of kCsrBlockLanes threads each
 constexpr int kCsrBlockLanes = 256;
-inline int csr_lanes(int64_t nnz, int64_t n) {
+// FP64 handles: 8 lanes when the rows give 8 resident warps an SM that way,
+// else 16, else 32.  There the FP64 pipe bounds the product (16 clocks a warp
+// instruction), and a row of 70 entries takes 3 adds by entries and 5 in the
+// butterfly with a warp to itself, (9 + 3) / 4 with 8 lanes (measured, FP64
+// elliptic ms of a step, 32 or 16 lanes / this rule: slab 51x51x26 3.85 / 3.46,
+// 101x101x26 10.5 / 8.3, 121x121x41 18.5 / 13.0; all at 4: 3.79, 11.6, -).
+inline int csr_lanes(int64_t nnz, int64_t n, bool f64) {
   if (n > 0 && nnz >= 256 * n) return kCsrBlockLanes;
+  if (f64 && nnz > 16 * n) {
+    int l = 8;
+    while (l < 32 && l * n < 152 * 8 * 32) l *= 2;
+    return l;
+  }
   const int64_t q = n > 0 ? (nnz + 4 * n - 1) / (4 * n) : 1;
   int l = 4;
   while (l < 32 && l < q) l *= 2;
@@ -454,6 +470,8 @@ struct StreamLaunch {
   long long* launch_acc;          // kernels launched (counted on the device)
   const int* gate;                // optional: the solve is skipped when *gate == 0
   int grid;                       // blocks of the row kernels (capped at a multiple of the SMs)
+  int strict;                     // 1: failures as the persistent FP64 kernel reports and leaves them: a
+                                  // breakdown is ST_INDEFINITE, and x keeps the updates made before it
   int host_loop;                  // 1: the loops run on the host (eager launches, no graph conditions)
   // optional SELL-32/4 copy of the inner operator (FP32 only; see launch_sell_v4):
   // used by the Krylov product and by the AMG level-0 products, whose operator

@@ -514,7 +514,7 @@ template <class T, class S>
 __global__ void __launch_bounds__(kSB) st_xupdate_kernel(const __grid_constant__ S src) {
   SEG_BEGIN(src)
   const StreamScal& c = *a.sc;
-  if (!c.inner_ran || c.fail) return;
+  if (!adds_correction(a)) return;
   const double s = c.scale;
   const T* d = static_cast<const T*>(a.d);
   for (int i = gt; i < a.n; i += gs) a.x[i] += s * double(d[i]);

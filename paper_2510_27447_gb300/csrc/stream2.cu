@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(kSB) st2_xupdate_kernel(const __grid_constant_
   PAIR_BEGIN(P)
   const StreamScal& c0 = *P.a[0].sc;
   const StreamScal& c1 = *P.a[1].sc;
-  by_mask(c0.inner_ran && !c0.fail, c1.inner_ran && !c1.fail, [&](auto m) {
+  by_mask(adds_correction(P.a[0]), adds_correction(P.a[1]), [&](auto m) {
     MASK_OF(m);
     const double s[2] = {c0.scale, c1.scale};
     for (int i = gt; i < a.n; i += gs)

@@ -376,12 +376,18 @@ __device__ __forceinline__ bool pq_decide(const StreamLaunch& a, T pq) {
   StreamScal& c = *a.sc;
   if (!(pq > T(0))) {
     if (!isfinite(pq)) c.fail |= ST_NONFINITE;
+    else if (a.strict) c.fail |= ST_INDEFINITE;
     c.stop = 1;
     c.inner_total += c.it;
     return false;
   }
   c.alpha = double(T(c.rho) / pq);
   return true;
+}
+
+// does the pass just run add its correction to x?
+__device__ __forceinline__ bool adds_correction(const StreamLaunch& a) {
+  return a.sc->inner_ran && !(a.strict ? a.sc->fail & ST_NONFINITE : a.sc->fail);
 }
 
 }  // namespace
