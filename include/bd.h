@@ -151,8 +151,8 @@ typedef struct {
                             streaming handle's parabolic solves are persistent below 7M entries, a
                             persistent handle's elliptic solves run as kernel chains inside its
                             captured steps (use_graph) where those are faster: 3-D meshes,
-                            FP64 sheets of more than 77,824 nodes, mixed-precision sheets of
-                            more than 1M entries */
+                            FP64 two-system solves and sheets of more than 77,824 nodes, mixed-
+                            precision sheets of more than 1M entries */
   int vec4;              /* 0 (default): mixed-precision streaming solves also keep the FP32
                             elliptic and parabolic operators, and every FP32 AMG level operator
                             stored as SELL-32 with at least 2^17 rows, in the SELL-32/4 layout

@@ -67,14 +67,17 @@ static __device__ __align__(256) double g_noalloc_scratch[kNoAllocWords];
 // Measured, elliptic ms of a step persistent / chain, one solve (1 sweep) and
 // one + pair (2 sweeps):
 //   FP64   slab  31x31x8  1.37 / 0.76, 4.09 / 1.84;  101x101x26 4.38 / 3.37,
-//          12.7 / 8.30;  sheet 257^2 0.92 / 1.19, 2.68 / 2.86;  285^2 1.55 /
-//          1.45, 4.51 / 3.50;  513^2 2.45 / 1.95, 7.23 / 4.79
+//          12.7 / 8.30;  sheet 129^2 0.76 / 0.87, 2.21 / 2.08;  257^2 0.92 /
+//          1.19, 2.68 / 2.86;  285^2 1.55 / 1.45, 4.51 / 3.50;  513^2 2.45 /
+//          1.95, 7.23 / 4.79
 //   mixed  slab 61x61x9   1.32 / 1.17, 2.98 / 2.48;  101x101x26 3.36 / 2.24,
 //          7.63 / 5.00;  sheet 257^2 0.69 / 1.04, 1.59 / 2.22;  401^2 1.37 /
 //          1.46, 3.38 / 3.15;  513^2 1.65 / 1.72, 3.97 / 3.57;  701^2 2.96 / 2.20
-// So: 3-D patterns always; 2-D ones in FP64 where the rows leave the
-// 512-thread build (77,824 = 152 x 512 rows), in mixed precision the pair from
-// 1M entries and the single solve from 2.5M.
+// So: FP64 pairs always (the persistent form solves one after the other: 2 x
+// 0.88 against 1.67 on the 257^2 sheet); 3-D patterns always; 2-D single solves
+// in FP64 where the rows leave the 512-thread build (77,824 = 152 x 512 rows);
+// in mixed precision, 2-D, the pair from 1M entries and the single solve from
+// 2.5M.
 struct ChainRule {
   bool one = false, two = false;
 };
@@ -88,7 +91,8 @@ static ChainRule chain_rule(const bd_opts_t& o, int64_t N, int64_t nnz) {
     r.one = rows3d || nnz >= 2500000;
     r.two = rows3d || nnz >= 1000000;
   } else {
-    r.one = r.two = rows3d || N > 152 * 512;
+    r.one = rows3d || N > 152 * 512;
+    r.two = true;
   }
   return r;
 }

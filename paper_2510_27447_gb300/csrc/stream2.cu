@@ -107,7 +107,7 @@ __device__ __forceinline__ void srow_m(const int64_t* __restrict__ sptr, const i
   const int w = sw[s];
   acc[0] = X(0);
   acc[1] = X(0);
-  constexpr int CH = 4;
+  constexpr int CH = kRowChunk<STREAMOP, V>;
   int c[CH];
   V v[CH];
   auto load = [&](int k0, int (&cc)[CH], V (&vv)[CH]) {

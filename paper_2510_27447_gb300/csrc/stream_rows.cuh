@@ -38,7 +38,15 @@ __device__ __forceinline__ V ld_stream(const V* p) {
 }
 
 // sum_k val[k] x[col[k]] over row i of a SELL-32 operator, entries in order,
-// four loads of each stream in flight per thread
+// four loads of each stream in flight per thread; eight on the coarse levels in
+// FP64, whose rows leave most of an SM's warps empty (elliptic ms of a step, one
+// solve / pair, 4 -> 8: slab 101x101x26 3.40 / 5.14 -> 3.12 / 4.93, sheet 401^2
+// 1.58 / 2.40 -> 1.53 / 2.17; 16: 3.29 / 5.79).  In FP32 eight gain nothing
+// (slab 161x161x41 5.37 / 6.42 -> 5.27 / 6.47, sheet 513^2 1.69 / 1.79 -> 1.77 /
+// 1.71); on level 0 in FP64 they trade threads for loads and gain on slabs what
+// they lose on sheets.
+template <bool STREAMOP, class V>
+constexpr int kRowChunk = !STREAMOP && sizeof(V) == 8 ? 8 : 4;
 template <bool STREAMOP, class V, class X>
 __device__ __forceinline__ X srow(const int64_t* __restrict__ sptr, const int* __restrict__ sw,
                                   const int* __restrict__ col, const V* __restrict__ val, const X* __restrict__ x,
@@ -47,7 +55,7 @@ __device__ __forceinline__ X srow(const int64_t* __restrict__ sptr, const int* _
   const int64_t base = sptr[s] + (i & 31);
   const int w = sw[s];
   X acc = X(0);
-  constexpr int CH = 4;
+  constexpr int CH = kRowChunk<STREAMOP, V>;
   for (int k0 = 0; k0 < w; k0 += CH) {
     int c[CH];
     V v[CH];

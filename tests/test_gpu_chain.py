@@ -34,7 +34,7 @@ def _run(w, M, K, steps=2, **opt):
 # mesh, precision, whether single and two-system solves become chains
 CASES = [(("slab", 31, 31, 8), binding.FP64, True, True), (("slab", 41, 37, 12), binding.MIXED, True, True),
          (("sheet", 281), binding.FP64, True, True), (("bath", 281), binding.FP64, True, True),
-         (("sheet", 277), binding.FP64, False, False), (("sheet", 385), binding.MIXED, False, True),
+         (("sheet", 277), binding.FP64, False, True), (("sheet", 385), binding.MIXED, False, True),
          (("sheet", 375), binding.MIXED, False, False)]
 
 
