@@ -366,14 +366,16 @@ float* p_values_f(bd_state* s, double alpha) {
   if (!dv || !alloc_n(s, &v, s->ell_n)) return nullptr;
   if (launch_to_float(s->ell_n, dv, v, s->stream) != cudaSuccess) return nullptr;
   float* v4 = nullptr;
-  if (s->vec4 && (!alloc_n(s, &v4, s->ell_n4) ||
-                  launch_sell_v4(s->n_slices, s->sptr, s->swidth, s->sptr4, v, v4, s->stream) != cudaSuccess))
+  if (s->vec4 && s->streaming && (!alloc_n(s, &v4, s->ell_n4) ||
+                                  launch_sell_v4(s->n_slices, s->sptr, s->swidth, s->sptr4, v, v4, s->stream) !=
+                                      cudaSuccess))
     return nullptr;
   s->fpcache.push_back({alpha, v, v4});
   return v;
 }
 
-// the SELL-32/4 copy of p_values_f(s, alpha) (NULL without vec4)
+// the SELL-32/4 copy of p_values_f(s, alpha) (NULL without vec4 and on persistent handles, whose
+// kernel chains are elliptic only)
 float* p_values_f4(bd_state* s, double alpha) {
   if (!p_values_f(s, alpha)) return nullptr;
   for (auto& pc : s->fpcache)

@@ -107,3 +107,37 @@ def test_step_in_a_callers_capture():
     v, u, X = sim.fields(full=True)
     sim.close()
     assert rel(X, ref[2]) < 1e-9 and rel(u, ref[1]) < 1e-9
+
+
+@pytest.mark.parametrize("mesh,prec", [(("slab", 31, 31, 8), binding.FP64), (("slab", 41, 37, 12), binding.MIXED)])
+def test_batches_are_untouched(mesh, prec):
+    w = _mesh(*mesh)
+    out = []
+    for s in (0, -1):
+        sims = [gpu_sim(w, precision=prec, streaming=s) for _ in range(2)]
+        for k, sim in enumerate(sims):
+            sim.set_initial(rest_X(w) * (1.0 + 0.001 * k))
+        for _ in range(2):
+            binding.batch_step(sims, w.dt, 3, 2)
+        out.append([a for sim in sims for a in sim.fields(full=True)])
+        for sim in sims:
+            sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", [binding.FP64, binding.MIXED])
+def test_footprint_holds_the_chains(prec):
+    torch = pytest.importorskip("torch")
+    w = W.config2(101, 101, 26)
+    opts = binding.default_options(pin_node=w.pin_node, precision=prec)
+    est = binding.footprint_bytes(w.xyz, w.elems, w.model, opts, w.elem_bath)
+    torch.cuda.init()
+    torch.cuda.synchronize()
+    free0, _ = torch.cuda.mem_get_info()
+    sim = binding.simulation_from_workload(w, opts)
+    sim.step(w.dt, 3, 2)
+    sim.sync()
+    free1, _ = torch.cuda.mem_get_info()
+    sim.close()
+    assert 0.9 < est / (free0 - free1) < 1.6   # the bounds of the other forms' test
