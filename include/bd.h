@@ -155,7 +155,8 @@ typedef struct {
                             precision sheets of more than 1M entries */
   int vec4;              /* 0 (default): mixed-precision streaming solves also keep the FP32
                             elliptic and parabolic operators, and every FP32 AMG level operator
-                            stored as SELL-32 with at least 2^17 rows, in the SELL-32/4 layout
+                            stored as SELL-32 with at least 2^15 rows (persistent
+                            handles, elliptic chains: 2^17), in the SELL-32/4 layout
                             (four consecutive entries of a row per 16-byte load; 8 more bytes
                             per stored entry) and use it in their products; 1: the same for
                             every SELL-32 level operator whatever its size (testing); -1: none
@@ -169,7 +170,7 @@ typedef struct {
                             every CSR level (tuning and testing); BD_ERR_ARG otherwise */
   int wide_sell;         /* streaming handles, AMG levels with rows longer than 32 entries: 0
                             (default) SELL-32 (thread per row) when padding stores at most 1.5x
-                            the entries and the level has at least 2^17 rows averaging at most 96
+                            the entries and the level has at least 2^15 rows averaging at most 96
                             entries, else CSR; 1: SELL-32 whenever the padding allows; -1:
                             always CSR; BD_ERR_ARG otherwise */
   int pair_solve;        /* AMG-preconditioned elliptic solves: the two elliptic solves of

@@ -406,7 +406,7 @@ SellHost sell_from_csr(const HCsr& A, int wide) {
       padded += 32 * w;
     }
     const int64_t nnz = A.rp[A.n];
-    sell_wide = 2 * padded <= 3 * nnz && (wide == 2 || (nnz <= 96 * A.n && A.n >= (int64_t(1) << 17)));
+    sell_wide = 2 * padded <= 3 * nnz && (wide == 2 || (nnz <= 96 * A.n && A.n >= kWideSellRows));
   }
   if (maxw > 32 && !sell_wide) {
     // long rows (coarse operators, restrictions in 3-D): CSR, one warp per row

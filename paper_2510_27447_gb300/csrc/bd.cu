@@ -1043,9 +1043,10 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH, bool built) {
       out->sw = csr ? nullptr : static_cast<const int*>(upload(S.sw.data(), S.sw.size() * 4));
       out->col = static_cast<const int*>(upload(S.col.data(), S.col.size() * 4));
       out->val = static_cast<const float*>(upload(fv.data(), fv.size() * 4));
-      // SELL-32/4 copy for the streaming kernels: operators of at least 2^17
-      // rows (vec4 = 0) or every SELL operator (vec4 = 1)
-      const bool v4 = !csr && s->vec4 && (s->opts.vec4 == 1 || S.n >= (int64_t(1) << 17));
+      // SELL-32/4 copy for the streaming kernels: operators of at least
+      // kWideSellRows rows (persistent handles, elliptic chains: 2^17), or every
+      // SELL operator (vec4 = 1)
+      const bool v4 = !csr && s->vec4 && (s->opts.vec4 == 1 || S.n >= (s->streaming ? kWideSellRows : int64_t(1) << 17));
       std::vector<int64_t> p4;
       std::vector<int> c4;
       std::vector<float> f4;

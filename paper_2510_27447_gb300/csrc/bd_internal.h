@@ -304,8 +304,13 @@ struct SellHost {
 // SELL-32 for rows of at most 32 entries, else CSR.  For operators only the
 // streaming kernels read, wide > 0 also allows SELL-32 for longer rows when
 // padding stores at most 1.5x the entries (SellHost.wmax = 0 then): wide = 1
-// only for operators of at least 2^17 rows averaging at most 96 entries,
+// only for operators of at least kWideSellRows rows averaging at most 96 entries,
 // wide = 2 whenever the padding allows
+// (the line: elliptic ms of a step, one solve / pair, with 2^17 and 2^15 rows: slab
+// 121x121x26 mixed, 50,000 rows, 2.88 / 3.94 and 2.60 / 3.29; 121x121x41, 73,000,
+// 3.67 / 4.77 and 3.38 / 4.00, FP64 4.86 / 8.14 and 4.69 / 7.42; operators of 14,000
+// rows and fewer lose)
+constexpr int64_t kWideSellRows = int64_t(1) << 15;
 SellHost sell_from_csr(const HCsr& A, int wide = 0);
 
 constexpr int kMaxAmgLevels = 10;
