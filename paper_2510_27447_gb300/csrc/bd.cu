@@ -1496,7 +1496,10 @@ struct BatchPlan {
   std::vector<bd_state*> m;
   cudaStream_t side[2] = {nullptr, nullptr};
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};   // launches side by side within a capture
+  // launches side by side within a capture; streams of their own, since `side`
+  // captures loop bodies and may not be part of another capture then
+  cudaStream_t fork[2] = {nullptr, nullptr};
+  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
   BatchCtl* ctl = nullptr;
   // arena chunks (one per captured step shape; graphs keep pointing into theirs)
   std::vector<char*> chunks;
@@ -1517,7 +1520,7 @@ struct BatchPlan {
     for (auto& g : graphs) cudaGraphExecDestroy(g.exec);
     for (char* c : chunks) cudaFree(c);
     if (ctl) cudaFree(ctl);
-    for (cudaStream_t x : side)
+    for (cudaStream_t x : {side[0], side[1], fork[0], fork[1]})
       if (x) cudaStreamDestroy(x);
     if (ev_in) cudaEventDestroy(ev_in);
     if (ev_out) cudaEventDestroy(ev_out);
@@ -1635,13 +1638,13 @@ int batch_solve_resident(BatchPlan& B, const BatchSolveArgs& q, cudaStream_t st,
   if (groups.size() > 1) BCK(cudaEventRecord(B.ev_fork, st));
   for (size_t k = 0; k < groups.size(); ++k) {
     const Group& g = groups[k];
-    const cudaStream_t to = k == 0 ? st : B.side[(k - 1) % 2];
+    const cudaStream_t to = k == 0 ? st : B.fork[(k - 1) % 2];
     if (k > 0 && k <= 2) BCK(cudaStreamWaitEvent(to, B.ev_fork, 0));
     B.enq += 1;
     BCK(res_solve(g.shape, mixed, g.amg, nullptr, int(g.tab.size()), put(B, g.tab), g.smem, to));
   }
   for (size_t k = 0; k < 2 && k + 1 < groups.size(); ++k) {
-    BCK(cudaEventRecord(B.ev_join[k], B.side[k]));
+    BCK(cudaEventRecord(B.ev_join[k], B.fork[k]));
     BCK(cudaStreamWaitEvent(st, B.ev_join[k], 0));
   }
   return BD_OK;
@@ -2524,8 +2527,8 @@ int bd_batch_step(bd_state_t* const* states, int n, double dt, int M, int K) {
     auto P = std::make_unique<BatchPlan>();
     P->m.assign(states, states + n);
     if (cudaSetDevice(s0->device) != cudaSuccess) return fail(s0, BD_ERR_CUDA, "cudaSetDevice failed");
-    for (cudaStream_t& x : P->side)
-      if (cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking) != cudaSuccess)
+    for (cudaStream_t* x : {&P->side[0], &P->side[1], &P->fork[0], &P->fork[1]})
+      if (cudaStreamCreateWithFlags(x, cudaStreamNonBlocking) != cudaSuccess)
         return fail(s0, BD_ERR_CUDA, "batch stream creation failed");
     if (cudaEventCreateWithFlags(&P->ev_in, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&P->ev_out, cudaEventDisableTiming) != cudaSuccess ||

@@ -81,3 +81,23 @@ def test_iteration_cap_and_zero_right_hand_side():
     u, it = sim.solve_elliptic(np.zeros(w.n_nodes))
     assert it == 0 and not np.any(u)
     sim.close()
+
+
+@pytest.mark.parametrize("prec", [binding.FP64, binding.MIXED])
+def test_batch_of_clusters_and_chains(prec):
+    """Members of two cluster shapes and one that does not fit a cluster, in one
+    captured step: each gives the bits of a batch of its own."""
+    ws = [W.sheet(n, 0.02 * (n - 1), W.LR91, 0.02, 4, strip=0.06) for n in (33, 65, 129, 161)]
+
+    def run(group):
+        sims = [gpu_sim(w, precision=prec) for w in group]
+        for _ in range(2):
+            binding.batch_step(sims, 0.02, 3, 2)
+        out = [sim.fields(full=True) for sim in sims]
+        for sim in sims:
+            sim.close()
+        return out
+
+    for w, f in zip(ws, run(ws)):
+        for a, b in zip(f, run([w])[0]):
+            assert np.array_equal(a, b)
