@@ -22,7 +22,7 @@ LIB = os.path.join(LIBDIR, "libbd.so")
 SOURCES = ["bd.cu", "ionic.cu", "pcg.cu", "amg.cu", "mixed.cu", "stream.cu", "stream2.cu", "resident.cu", "assemble.cpp", "amg.cpp",
            "resident_plan.cpp"]
 HEADERS = ["bd_internal.h", "models.cuh", "sd.cuh", "sparse.cuh", "vcycle.cuh", "segment.cuh", "stream_rows.cuh",
-           "resident.h", "fixexp.h"]
+           "resident.h", "resident_order.h", "fixexp.h"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 NVCC_FLAGS = ["-O3", "-std=c++20", ARCH, "-lineinfo", "-Xcompiler", "-fPIC,-O3",
               "--expt-relaxed-constexpr", "-I" + os.path.join(ROOT, "include")]

@@ -18,11 +18,13 @@
 // store, its acknowledgement and a cluster barrier (measured, 16 blocks: 425
 // against 1,020 clocks).  Dot products travel the same way: partial sums go to
 // every block, and all add them in the same order.
-//   A buffer is sent to again only after a phase in which every block hears
-// from every other (a dot product, or the coarse gather, which carries a
-// token of each block for this) has completed at the sender: by then the
-// receiver has read it.  Phases that repeat without another such phase between
-// them (the pipelined loop) use two buffers and two mbarriers in turn.
+//   A buffer is sent to again, and an mbarrier counted on again, only after
+// another phase in which every block hears from every other (a dot product, or
+// the coarse gather, which carries a token of each block for this) has completed
+// at the sender: every block sent in it after reading the buffer.  A phase of
+// this kind does not protect its own buffer, so dot products use two buffers
+// and two mbarriers in turn (SumTurns), and so do the halos that travel with
+// them in the pipelined loop.
 //   Waits for peers are bounded (kWaitLimitNs): on expiry a warp records
 // ST_TIMEOUT and ends, except the block's first, which leaves through the
 // cluster barrier at the kernel's end so that no block is gone while a peer may
@@ -56,6 +58,7 @@
 #include <algorithm>
 
 #include "resident.h"
+#include "resident_order.h"
 #include "sparse.cuh"
 
 namespace bd {
@@ -68,9 +71,6 @@ struct ResPair {
 
 __host__ __device__ constexpr size_t up16(size_t v) { return (v + 15) & ~size_t(15); }
 
-// phases (one mbarrier each); levels l >= 1 have four: pre-smoothed x,
-// residual, corrected x, result
-enum : int { kRed = 0, kRed2, kSum0, kSum1, kXF, kZ, kX0, kRes, kX0b, kBc, kXc, kPin, kLev };
 constexpr int kPhases = kLev + 4 * (kResLevels - 1);
 static_assert(kPhases <= 32, "the parities are the bits of one word");
 
@@ -79,9 +79,8 @@ static_assert(kPhases <= 32, "the parities are the bits of one word");
 struct ResMem {
   int img0, valA, x0, zr, xf, st, part, lv[kResLevels][3], bc, xc, imgA, total;   // lv: b, x, y
 };
-// partial sums: FP32 2 phases x (16 warps x 16 blocks) x float4, FP64 3 phases
-// x 3 values x (4 warps x 16 blocks)
-constexpr int kPartF = 2 * 16 * kResMaxCluster * 4, kPartD = 3 * 3 * 4 * kResMaxCluster;
+// partial sums of two turns: FP32 (16 warps x 16 blocks) x float4, FP64 3 values x (4 warps x 16 blocks)
+constexpr int kPartF = 2 * 16 * kResMaxCluster * 4, kPartD = 2 * 3 * 4 * kResMaxCluster;
 template <class S>
 __host__ __device__ __forceinline__ void res_mem(const S& s, int img0, int imgA, int block, int vb, bool amg,
                                                  ResMem* m) {
@@ -528,8 +527,9 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
   cluster_barrier();   // every block's mbarriers and buffers are ready for its peers
 
   // scalars of the block: s_d = mean of b, |b|^2, tol^2 |b|^2, scale, 1 / scale, inner target
-  int outer = 0, nsum = 0;
-  auto next_sum = [&] { return kSum0 + (nsum++ & 1); };
+  int outer = 0;
+  SumTurns turns, turns32;                  // FP64 sums (kSum0, kSum1), FP32 sums (kRed, kRed2)
+  auto next_sum = [&] { return kSum0 + turns.next(); };
   // thread 0: what to do with the outer residual (s_code: 0 solve, 1 non-finite, 2 done, 3 out of passes)
   auto decide = [&](double rr64) {
     s_code = 0;
@@ -835,11 +835,12 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
         }
         if (!first) ++it;
         if constexpr (F32) {
-          __syncthreads();   // every warp has read the totals of the last iteration
-          ph.expect(kRed, nparts * 16);
-          sum_f32_send(ph, kRed, 0, t3, partf, iC, irank, nw);
-          ph.wait(kRed);
-          sum_f32_get(0, t3, partf, nparts);
+          const int turn = turns32.next(), k = kRed + turn;
+          __syncthreads();   // the products' vector is read
+          ph.expect(k, nparts * 16);
+          sum_f32_send(ph, k, turn, t3, partf, iC, irank, nw);
+          ph.wait(k);
+          sum_f32_get(turn, t3, partf, nparts);
           if (!ph.ok) break;
           const T rz = t3[0], rr = t3[2];
           if (first) {
@@ -866,7 +867,8 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
         } else {
           double (&td)[3] = reinterpret_cast<double (&)[3]>(t3);
           // s_code: 0 go on, -1 converged, else the failure
-          sum_f64<3>(ph, kRed, 2, td, stage, partd, iC, irank, [&](const double (&t)[3]) {
+          const int k = next_sum();
+          sum_f64<3>(ph, k, k - kSum0, td, stage, partd, iC, irank, [&](const double (&t)[3]) {
             s_code = first ? (!(t[2] > s_d[2]) ? -1 : 0)   // includes b = 0
                      : !isfinite(t[2]) || !isfinite(t[0]) ? ST_NONFINITE
                      : t[2] <= s_d[2]                     ? -1
