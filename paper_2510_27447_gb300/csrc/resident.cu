@@ -25,10 +25,10 @@
 // this kind does not protect its own buffer, so dot products use two buffers
 // and two mbarriers in turn (SumTurns), and so do the halos that travel with
 // them in the pipelined loop.
-//   Waits for peers are bounded (kWaitLimitNs): on expiry a warp records
-// ST_TIMEOUT and ends, except the block's first, which leaves through the
-// cluster barrier at the kernel's end so that no block is gone while a peer may
-// still send to it (ended threads count as arrived at both kinds of barrier).
+//   Waits for peers are bounded (kWaitLimitNs).  On expiry a warp records
+// ST_TIMEOUT; the block's next barrier tells all its warps, which then leave
+// through the cluster barrier at the kernel's end, so that no block is gone
+// while a peer may still send to it (PhaseOrder).
 //
 // The iteration is the one of the grid kernels: Jacobi- or AMG-V(1,1)-
 // preconditioned CG; T = double solves in FP64, T = float is the mixed path's
@@ -72,7 +72,7 @@ struct ResPair {
 __host__ __device__ constexpr size_t up16(size_t v) { return (v + 15) & ~size_t(15); }
 
 constexpr int kPhases = kLev + 4 * (kResLevels - 1);
-static_assert(kPhases <= 32, "the parities are the bits of one word");
+static_assert(kPhases <= 29, "the parities and three flags are the bits of one word");
 
 // dynamic shared memory of a block: identical offsets in every block of the
 // cluster (a send addresses a peer's copy by the local offset)
@@ -143,43 +143,46 @@ __device__ __forceinline__ void cp_block(unsigned char* dst, const void* src, in
 }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// a thread's view of the block's phases: their mbarriers and parities
-struct Phases {
+// the block's mbarriers, its barrier and flags, as PhaseOrder uses them
+struct PhaseHw {
   unsigned mb;          // shared address of the mbarriers
-  unsigned par;         // parity of each phase's next completion
-  bool ok;              // no wait has run out (the same in all lanes of a warp)
   int* status;
 
   __device__ __forceinline__ unsigned addr(int k) const { return mb + 8u * unsigned(k); }
+  // (the two flags follow the mbarriers)
+  __device__ __forceinline__ int block_sync(bool late, bool turn) const {
+    const unsigned flag = addr(kPhases) + (turn ? 4u : 0u);
+    if (late) asm volatile("st.volatile.shared.u32 [%0], 1;" ::"r"(flag) : "memory");
+    __syncthreads();
+    int gone;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(gone) : "r"(flag) : "memory");
+    return gone;
+  }
   // the block expects bytes from its peers in phase k (thread 0, after a
   // barrier of the block behind the phase's own work)
-  __device__ __forceinline__ void expect(int k, int bytes) {
+  __device__ __forceinline__ void expect(int k, int bytes) const {
     if (threadIdx.x == 0)
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(addr(k)), "r"(bytes) : "memory");
   }
-  __device__ __forceinline__ void wait(int k) {
-    const unsigned p = par >> k & 1u;
-    par ^= 1u << k;
-    if (!ok) return;
+  // false (in all lanes of the warp) once kWaitLimitNs have passed
+  __device__ __forceinline__ bool await(int k, unsigned parity) const {
     unsigned long long t0 = 0;
-  #pragma unroll 1
+#pragma unroll 1
     for (unsigned n = 1;; ++n) {
       unsigned d;
       asm volatile(
           "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2;\n\t"
           "selp.u32 %0, 1, 0, q;\n\t}"
           : "=r"(d)
-          : "r"(addr(k)), "r"(p)
+          : "r"(addr(k)), "r"(parity)
           : "memory");
-      if (__all_sync(0xffffffffu, d != 0u)) return;
+      if (__all_sync(0xffffffffu, d != 0u)) return true;
       if ((n & 63u) == 0u) {
         const unsigned long long t = device_ns();
         if (t0 == 0) t0 = t;
         if (__any_sync(0xffffffffu, t - t0 > kWaitLimitNs)) {
           if ((threadIdx.x & 31) == 0) atomicOr(status, ST_TIMEOUT);
-          if (threadIdx.x >= 32) asm volatile("exit;");
-          ok = false;
-          return;
+          return false;
         }
       }
     }
@@ -206,24 +209,28 @@ struct Phases {
         : "memory");
   }
 };
+using Phases = PhaseOrder<PhaseHw>;
 
 // The owned entries of vec are written: send the peers theirs and wait for
 // the block's own halo (bytes: what the block expects in phase k besides)
 template <class T>
 __device__ __forceinline__ void exchange(Phases& ph, const uint32_t* word, int n, T* vec, int k, int bytes) {
-  __syncthreads();
+  if (!ph.ok()) return;
+  const int gone = ph.meet();
   ph.expect(k, bytes);
 #pragma unroll 1
   for (int e = opaque(threadIdx.x); e < n; e += blockDim.x) {
     const uint32_t w = word[e];
     ph.send(vec + (w & 0xffffu), w >> 16 & 15u, vec[w >> 20], k);
   }
+  ph.learn(gone);
   ph.wait(k);
 }
 // count values of a coarse vector, owned from c0 on (a multiple of 4), to every block
 template <class T>
 __device__ __forceinline__ void gather_all(Phases& ph, T* vec, int c0, int count, int C, int k, int bytes) {
-  __syncthreads();
+  if (!ph.ok()) return;
+  const int gone = ph.meet();
   ph.expect(k, bytes);
   const int sh = 31 - __clz(C);          // C is a power of two
   if constexpr (sizeof(T) == 4) {        // the padding entries travel along
@@ -239,6 +246,7 @@ __device__ __forceinline__ void gather_all(Phases& ph, T* vec, int c0, int count
       ph.send(p, unsigned(e & (C - 1)), *p, k);
     }
   }
+  ph.learn(gone);
   ph.wait(k);
 }
 
@@ -300,7 +308,8 @@ __device__ __forceinline__ void sum_f64(Phases& ph, int k, int part_slot, double
   double* pt = part + part_slot * 3 * 4 * kResMaxCluster;
 #pragma unroll
   for (int i = 0; i < NV; ++i) stage[i * bd + threadIdx.x] = v[i];
-  __syncthreads();
+  if (!ph.ok()) return;
+  const int gone = ph.meet();
   ph.expect(k, C * 4 * NV * 8);
   if (wid < 4) {
 #pragma unroll 1
@@ -313,6 +322,7 @@ __device__ __forceinline__ void sum_f64(Phases& ph, int k, int part_slot, double
       for (int c = lane & (G - 1); c < C; c += G)
         ph.send(pt + i * 4 * kResMaxCluster + rank * 4 + wid, unsigned(c), x, k);
   }
+  ph.learn(gone);
   ph.wait(k);
   if (wid == 0) {
     double p[NV];
@@ -325,9 +335,9 @@ __device__ __forceinline__ void sum_f64(Phases& ph, int k, int part_slot, double
     const double x = warp_sum_spread<NV>(p);
 #pragma unroll
     for (int i = 0; i < NV; ++i) p[i] = __shfl_sync(0xffffffffu, x, i * G);
-    if (lane == 0) f(p);
+    if (lane == 0 && !ph.late()) f(p);
   }
-  __syncthreads();
+  ph.sync();
 }
 
 // FP32 sums of three values over the cluster: every warp sends its partials
@@ -393,7 +403,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ __align__(16) ResLaunch a;
   __shared__ ResMem M;    // the level loops index it at run time
-  __shared__ __align__(8) unsigned long long s_mb[kPhases];
+  __shared__ __align__(8) unsigned long long s_mb[kPhases + 1];   // and the block's two flags
   __shared__ double s_pin, s_d[6];
   __shared__ int s_code;
   __shared__ float s_tok[kResMaxCluster];
@@ -411,6 +421,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
   if (a.gate && *a.gate == 0) return;   // the same in every block of the cluster
   if (tid == 0) res_mem(a, a.img0, a.imgA, bd, int(sizeof(T)), AMG, &M);
   if (tid < kPhases) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&s_mb[tid])), "r"(1));
+  if (tid == kPhases) s_mb[kPhases] = 0ull;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
   const ResCta ct = a.cta[rank];
@@ -421,7 +432,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
   // entry of a level never writes
   for (int i = M.zr + 16 * tid; i < M.imgA; i += 16 * bd) *reinterpret_cast<float4*>(sm + i) = make_float4(0.f, 0.f, 0.f, 0.f);
 
-  Phases ph{smem_addr(s_mb), 0u, true, a.status};
+  Phases ph{{smem_addr(s_mb), a.status}};
   const uint32_t* sl0 = reinterpret_cast<const uint32_t*>(sm + M.img0);
   const uint16_t* lcol = reinterpret_cast<const uint16_t*>(sm + M.img0 + a.off_lcol);
   const uint32_t* push0 = reinterpret_cast<const uint32_t*>(sm + M.img0 + a.off_push);
@@ -601,7 +612,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
       const int k = next_sum();
       sum_f64<1>(ph, k, k - kSum0, s1, stage, partd, iC, irank, [&](const double (&t)[1]) { decide(t[0]); });
     }
-    if (!ph.ok) break;
+    if (!ph.ok()) break;
     const int code = s_code;
     if (code != 0) {
       if (code == 1) fail = ST_NONFINITE;
@@ -645,7 +656,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
         float gam_prev = 1.f, alpha_prev = 1.f;
         for (;;) {
           const int odd = it & 1;
-          if (!ph.ok) break;
+          if (!ph.ok()) break;
           float t[3];
           sum_f32_get(odd, t, partf, nparts);
           const float gam = t[0], del = t[1], rr = t[2];
@@ -836,12 +847,14 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
         if (!first) ++it;
         if constexpr (F32) {
           const int turn = turns32.next(), k = kRed + turn;
-          __syncthreads();   // the products' vector is read
+          if (!ph.ok()) break;
+          const int gone = ph.meet();   // the products' vector is read
           ph.expect(k, nparts * 16);
           sum_f32_send(ph, k, turn, t3, partf, iC, irank, nw);
+          ph.learn(gone);
+          if (!ph.ok()) break;
           ph.wait(k);
           sum_f32_get(turn, t3, partf, nparts);
-          if (!ph.ok) break;
           const T rz = t3[0], rr = t3[2];
           if (first) {
             if (!(rr > target2)) break;      // includes b = 0
@@ -883,7 +896,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
               rho = t[0];
             }
           });
-          if (!ph.ok) break;
+          if (!ph.ok()) break;
           if (s_code != 0) {
             fail = s_code > 0 ? s_code : 0;
             break;
@@ -901,7 +914,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
       }
     }
     inner_total += it;
-    if ((fail && F32) || !ph.ok) break;
+    if ((fail && F32) || !ph.ok()) break;
 #pragma unroll
     for (int j = 0; j < RPT; ++j) xs[j] += F32 ? scale * double(d[j]) : double(d[j]);
     if (!F32 || a.max_outer == 1) break;
@@ -930,7 +943,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
                [&](const double (&t)[1]) { s_d[0] = t[0] / double(a.n); });
     shift = s_d[0];
   }
-  if (ph.ok) {
+  if (ph.sync()) {
 #pragma unroll
     for (int j = 0; j < RPT; ++j)
       if (tid + j * bd < nloc) a.x[r0 + tid + j * bd] = xs[j] - shift;
