@@ -167,14 +167,37 @@ BD_FIX_FN double exp_fixed(double x) {
 #endif
 }
 
-// 1 / d in integer arithmetic: the mantissa's reciprocal from FP32 (24 bits) by
-// two Newton steps r += r (1 - m r) in 64 bits, rounded once: at most 0.501
-// units in the last place (tests/test_exp_cpu.py).  Zero, subnormal and
-// non-finite d, and d whose reciprocal is subnormal, take the division.
+// 1 / d in integer arithmetic, correctly rounded as the division is: the
+// mantissa's reciprocal from FP32 by two Newton steps r += r (1 - m r) in 64
+// bits, cut to 53 bits, and the rounding decided by the sign of an exact
+// product.  Zero, subnormal and non-finite d, and d whose reciprocal is
+// subnormal, take the division.
+//   Seed: m cut to 24 bits (below 2^-23 relative) and __fdividef (2 units in the
+// last place, 2^-22 relative), so |1 - m r0| < 1.5 2^-21 and the 52-bit e1 is
+// below 2^30 after its shift; the first step leaves 2^-41, the second what its
+// truncations do (a few units of 2^-64, where rounding bears 2^10).
+//   Measured on GB300, FP64 steps, with the rounding of r itself (0.501 units in
+// the last place) / this: TP06 257^2 7.22 / 7.28 ms, slab 101x101x26 20.5 / 20.7.
 #ifdef __CUDACC__
 __host__ __device__ __noinline__
 #endif
 inline double recip_outside(double d) { return 1.0 / d; }
+
+// bits: a normal d with a normal reciprocal; r0: the reciprocal of its mantissa, at 2^32
+BD_FIX_FN uint64_t recip_from_seed(uint64_t bits, uint32_t r0) {
+  const uint64_t m = bits << 11 | 0x8000000000000000ull;               // m / 2^63 in [1, 2)
+  const int64_t e1 = int64_t(0x8000000000000000ull - fix_mulhi(m, uint64_t(r0) << 32));   // (1 - m r0) 2^63
+  const uint64_t r1 = (uint64_t(r0) << 32) + uint64_t((int64_t(r0) * int64_t(int32_t(e1 >> 12))) >> 19);
+  const int64_t e2 = int64_t(0x8000000000000000ull - fix_mulhi(m, r1));
+  uint64_t r2 = r1 + uint64_t((int64_t(r1 >> 32) * e2) >> 31);
+  if (e2 > 0 && r2 < r1) r2 = ~uint64_t(0);                             // m = 1: rounded up to 2^64
+  // 1/m lies above q + 1/2 where (2 q + 1) m < 2^106; the product is within 2^55
+  // of 2^106, so its low 64 bits have the difference's sign
+  const uint64_t q = r2 >> 11;
+  const int64_t side = int64_t((2 * q + 1) * (m >> 11));
+  return q + (side < 0 ? 1u : 0u) + (uint64_t(2044u - (uint32_t(bits >> 52) & 0x7ffu)) << 52) +
+         (bits & 0x8000000000000000ull);
+}
 
 BD_FIX_FN double recip_fixed(double d) {
   uint64_t bits;
@@ -185,9 +208,8 @@ BD_FIX_FN double recip_fixed(double d) {
 #endif
   const uint32_t be = uint32_t(bits >> 52) & 0x7ffu;
   if (be - 1u >= 2043u) return recip_outside(d);
-  const uint64_t m = bits << 11 | 0x8000000000000000ull;               // m / 2^63 in [1, 2)
-  uint32_t r0;                                                          // reciprocal, 2^32
-  const uint32_t fb = 0x3f800000u | (uint32_t(m >> 40) & 0x7fffffu);
+  uint32_t r0;
+  const uint32_t fb = 0x3f800000u | (uint32_t(bits >> 29) & 0x7fffffu);
 #ifdef __CUDA_ARCH__
   r0 = __float2uint_rz(__fdividef(1.0f, __uint_as_float(fb)) * 4294967296.0f);   // saturates at 2^32 - 1
 #else
@@ -196,12 +218,7 @@ BD_FIX_FN double recip_fixed(double d) {
   const float r = 1.0f / f * 4294967296.0f;
   r0 = r >= 4294967296.0f ? 0xffffffffu : uint32_t(r);
 #endif
-  const int64_t e1 = int64_t(0x8000000000000000ull - fix_mulhi(m, uint64_t(r0) << 32));   // (1 - m r0) 2^63
-  const uint64_t r1 = (uint64_t(r0) << 32) + uint64_t((int64_t(r0) * int64_t(int32_t(e1 >> 11))) >> 20);
-  const int64_t e2 = int64_t(0x8000000000000000ull - fix_mulhi(m, r1));
-  uint64_t r2 = r1 + uint64_t((int64_t(r1 >> 32) * e2) >> 31);
-  if (e2 > 0 && r2 < r1) r2 = ~uint64_t(0);                             // m = 1: rounded up to 2^64
-  const uint64_t out = (r2 >> 11) + (r2 >> 10 & 1) + (uint64_t(2044u - be) << 52) + (bits & 0x8000000000000000ull);
+  const uint64_t out = recip_from_seed(bits, r0);
 #ifdef __CUDA_ARCH__
   return __longlong_as_double((long long)out);
 #else
