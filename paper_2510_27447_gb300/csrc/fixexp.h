@@ -228,4 +228,8 @@ BD_FIX_FN double recip_fixed(double d) {
 #endif
 }
 
+// Jacobi scaling 1 / d of a row, rounded to T once, without the FP64 pipe
+template <class T>
+BD_FIX_FN T jacobi_scale(double d) { return T(recip_fixed(d)); }
+
 }  // namespace bd

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(TPB, MINB) pcg_mixed_kernel(const __grid_const
     m.b64[i] = b;
     double d = a.valA[a.diagpos[i]];
     if (a.dextra) d += a.dextra[i];
-    m.invd32[i] = 1.0f / float(d);
+    m.invd32[i] = jacobi_scale<float>(d);
     acc0[0] += b;
     acc0[1] += b * b;
     if (fused) {

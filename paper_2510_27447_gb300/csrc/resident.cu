@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
         if (a.val1) bi += a.c1 * sp[0];
         if (a.val2) bi += a.c2 * sp[1];
         const double de = a.dextra ? a.dextra[i] : 0.0;
-        invd[j] = T(1) / T(a.valA[a.diagpos[i]] + de);
+        invd[j] = jacobi_scale<T>(a.valA[a.diagpos[i]] + de);
         dx[j] = T(de);
         double ri = bi;
         if (a.warm) {

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "bd_internal.h"
+#include "fixexp.h"
 
 namespace bd {
 

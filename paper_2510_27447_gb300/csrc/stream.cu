@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kSB) st_rhs_kernel(const __grid_constant__ S s
     if (!a.use_amg) {
       double d = a.valA[a.diagpos[i]];
       if (a.dextra) d += a.dextra[i];
-      invd[i] = T(1) / T(d);   // FP32: no FP64 division per row
+      invd[i] = jacobi_scale<T>(d);
     }
     if (!a.warm) a.x[i] = 0.0;
     acc[0] += b;
