@@ -264,6 +264,31 @@ bool dense_spd_inverse(std::vector<double>& a, int64_t n, std::vector<double>* i
   return true;
 }
 
+// the coarsest level of a hierarchy: dense inverse of A_c + c 1 1^T
+int coarse_inverse(const HCsr& A, AmgHost* out, std::string* err) {
+  const int64_t n = A.n;
+  if (n > 4096) {
+    *err = "AMG: coarsest level too large for a dense solve";
+    return BD_ERR_ARG;
+  }
+  std::vector<double> dense(n * n, 0.0);
+  double dmean = 0.0;
+  for (int64_t i = 0; i < n; ++i)
+    for (int64_t p = A.rp[i]; p < A.rp[i + 1]; ++p) {
+      dense[i * n + A.ci[p]] += A.v[p];
+      if (A.ci[p] == i) dmean += A.v[p];
+    }
+  dmean /= double(std::max<int64_t>(n, 1));
+  const double c = dmean / double(std::max<int64_t>(n, 1));
+  for (auto& x : dense) x += c;
+  if (!dense_spd_inverse(dense, n, &out->cinv)) {
+    *err = "AMG: coarsest operator is not positive definite";
+    return BD_ERR_ARG;
+  }
+  out->nc = n;
+  return BD_OK;
+}
+
 }  // namespace
 
 int amg_build(const HCsr& A0, const AmgParams& prm, AmgHost* out, std::string* err) {
@@ -357,28 +382,16 @@ int amg_build(const HCsr& A0, const AmgParams& prm, AmgHost* out, std::string* e
     out->lev.push_back(std::move(L));
     A = std::move(Ac);
   }
-  // coarsest operator: dense inverse of A_c + c 1 1^T
-  const int64_t n = A.n;
-  if (n > 4096) {
-    *err = "AMG: coarsest level too large for a dense solve";
-    return BD_ERR_ARG;
-  }
-  std::vector<double> dense(n * n, 0.0);
-  double dmean = 0.0;
-  for (int64_t i = 0; i < n; ++i)
-    for (int64_t p = A.rp[i]; p < A.rp[i + 1]; ++p) {
-      dense[i * n + A.ci[p]] += A.v[p];
-      if (A.ci[p] == i) dmean += A.v[p];
-    }
-  dmean /= double(std::max<int64_t>(n, 1));
-  const double c = dmean / double(std::max<int64_t>(n, 1));
-  for (auto& x : dense) x += c;
-  if (!dense_spd_inverse(dense, n, &out->cinv)) {
-    *err = "AMG: coarsest operator is not positive definite";
-    return BD_ERR_ARG;
-  }
-  out->nc = n;
-  return BD_OK;
+  return coarse_inverse(A, out, err);
+}
+
+int amg_truncate(int64_t coarse_max, AmgHost* H, std::string* err) {
+  size_t l = 1;
+  while (l < H->lev.size() && H->lev[l].A.n > coarse_max) ++l;
+  if (l >= H->lev.size()) return BD_OK;
+  const HCsr A = std::move(H->lev[l].A);
+  H->lev.resize(l);
+  return coarse_inverse(A, H, err);
 }
 
 }  // namespace bd

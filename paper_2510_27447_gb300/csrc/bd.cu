@@ -876,16 +876,22 @@ bool res_wanted(const bd_state* s) {
          s->opts.cg_grid == 0 && s->nnz * entry <= int64_t(kResMaxCluster) * 60 * 1024;
 }
 
-// Plan and upload the cluster-resident solves and leave their hierarchy in AH
-// (*built: it is); res_on stays false when the problem does not fit.
-// Hierarchy: coarsened to kResCoarseMax rows instead of AmgParams' 1500 (the
-// dense level's product runs on 16 SMs); in mixed precision also for meshes of
-// fewer than 1500 rows.  FP64 solves of those keep Jacobi: the tolerance bounds
-// the residual, and another preconditioner would move u by as much as it allows
-// (1e-9 of u at the default 1e-10).
-int setup_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sptr, const std::vector<int>& sw,
-                   AmgHost* AH, bool* built) {
-  *built = false;
+// the cluster-resident solves' host plan and hierarchy
+struct ResSetup {
+  bool fits = false;              // the handle's solves are cluster-resident
+  bool amg = false;               // the elliptic ones have a hierarchy
+  ResPlan P;
+  AmgHost AH;
+};
+
+// Plan the cluster-resident solves (on the host; the handle's other solver forms
+// are chosen by the outcome).  Hierarchy: coarsened to kResCoarseMax rows
+// instead of AmgParams' 1500 (the dense level's product runs on 16 SMs); in mixed
+// precision also for meshes of fewer than 1500 rows.  FP64 solves of those keep
+// Jacobi: the tolerance bounds the residual, and another preconditioner would
+// move u by as much as it allows (1e-9 of u at the default 1e-10).
+int plan_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sptr, const std::vector<int>& sw,
+                  ResSetup* R) {
   if (!res_wanted(s)) return BD_OK;
   const bool mixed = s->precision == BD_MIXED;
   AmgParams prm;
@@ -893,19 +899,28 @@ int setup_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sp
   else if (mixed || s->N > prm.coarse_max) prm.coarse_max = kResCoarseMax;
   if (s->opts.elliptic_precond == 1) {
     std::string err;
-    const int rc = amg_build(elliptic_csr(s, H), prm, AH, &err);
+    const int rc = amg_build(elliptic_csr(s, H), prm, &R->AH, &err);
     if (rc != BD_OK) return fail(s, rc, "%s", err.c_str());
   }
-  const AmgHost* hier = s->opts.elliptic_precond == 1 && !AH->lev.empty() ? AH : nullptr;
-  // the largest cluster the device schedules: measured (ms per step, 16 / 8
-  // blocks), LR91 65^2 FP64 2.07 / 2.64, TP06 129^2 mixed 1.85 / 2.37 (8 blocks do
-  // not hold it), LR91 33^2 mixed 0.68 / 0.69
-  ResPlan P;
-  bool fits = false;
-  for (int C = kResMaxCluster; C >= 8 && !fits; C /= 2)
-    fits = res_plan_build(C, s->N, H.rowptr.data(), H.col.data(), sptr.data(), sw.data(), hier, mixed, !mixed, &P) &&
-           res_prepare(P.s, mixed, false) && (!hier || res_prepare(P.s, mixed, true));
-  if (!fits) return BD_OK;
+  R->amg = !R->AH.lev.empty();
+  // the largest cluster the device schedules (a smaller one holds more per
+  // block): measured (ms per step, 16 / 8 blocks), LR91 65^2 FP64 2.07 / 2.64, TP06
+  // 129^2 mixed 1.85 / 2.37 (8 blocks do not hold it), LR91 33^2 mixed 0.68 / 0.69
+  for (int C = kResMaxCluster; C >= 8 && !R->fits; C /= 2) {
+    if (!res_plan_build(C, s->N, H.rowptr.data(), H.col.data(), sptr.data(), sw.data(), R->amg ? &R->AH : nullptr,
+                        mixed, !mixed, &R->P) ||
+        res_smem_bytes(R->P.s, mixed, R->amg) > kResSmemMax)
+      break;
+    R->fits = res_prepare(R->P.s, mixed, false) && (!R->amg || res_prepare(R->P.s, mixed, true));
+  }
+  return BD_OK;
+}
+
+// upload the plan; every solve of the handle takes it from here on
+int setup_resident(bd_state* s, const ResSetup& R) {
+  if (!R.fits) return BD_OK;
+  const bool mixed = s->precision == BD_MIXED;
+  const ResPlan& P = R.P;
   auto upload = [&](const void* h, size_t bytes) -> void* {
     void* d = dalloc(s, bytes);
     if (d && cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, s->stream) != cudaSuccess) return nullptr;
@@ -916,7 +931,7 @@ int setup_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sp
   s->res_g0 = static_cast<unsigned char*>(upload(P.img0.data(), P.img0.size()));
   bool ok = s->res_cta && s->res_g0;
   std::vector<float> ci32;
-  if (ok && hier) {
+  if (ok && R.amg) {
     const std::vector<unsigned char>& im = mixed ? P.imgA32 : P.imgA64;
     s->res_gA = static_cast<unsigned char*>(upload(im.data(), im.size()));
     if (mixed) ci32.assign(P.cinv.begin(), P.cinv.end());
@@ -926,25 +941,23 @@ int setup_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sp
   // a bath mesh's second system gathers its potential over all nodes too
   if (ok && s->NT < s->N && !s->vfull2)
     ok = alloc_n(s, &s->vfull2, s->N) && cudaMemsetAsync(s->vfull2, 0, s->N * 8, s->stream) == cudaSuccess;
-  // the plan's host arrays end here
+  // the host arrays of ci32 end here
   if (!ok || cudaStreamSynchronize(s->stream) != cudaSuccess) return fail(s, BD_ERR_OOM, "device allocation failed");
-  s->res_amg = hier != nullptr;
+  s->res_amg = R.amg;
   s->res_on = true;
-  *built = true;
   return BD_OK;
 }
 
 // build the AMG hierarchy of A_ie on the host and upload it (SELL-32 operators)
-// (built: AH holds the hierarchy of the cluster-resident solves, kept for meshes
-// that have one here too)
-int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH, bool built) {
+// (AH: the hierarchy planned for the cluster-resident solves, if any; kept when
+// they are taken, else its levels down to this one's coarsest)
+int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH) {
   std::string err;
   AmgParams prm;
   if (s->opts.amg_coarse_max > 0) prm.coarse_max = s->opts.amg_coarse_max;
   if (s->N <= prm.coarse_max) return BD_OK;   // small operator: Jacobi-PCG is used
-  if (!built) {
-    AH = AmgHost{};
-    const int rc = amg_build(elliptic_csr(s, H), prm, &AH, &err);
+  if (!s->res_on) {
+    const int rc = AH.lev.empty() ? amg_build(elliptic_csr(s, H), prm, &AH, &err) : amg_truncate(prm.coarse_max, &AH, &err);
     if (rc != BD_OK) return fail(s, rc, "%s", err.c_str());
   }
   if (AH.lev.empty()) return BD_OK;   // small operator: Jacobi-PCG is used
@@ -2278,8 +2291,16 @@ int bd_create(const bd_mesh_t* mesh, const bd_cond_t* cond, bd_ionic_t model, co
     s->streaming = s->opts.cg_cluster == 0 && (so >= 1 || (so == 0 && nnz >= kStreamNnz));
     s->stream_par = s->streaming && (so >= 1 || s->precision != BD_MIXED || nnz >= kStreamParNnz);
     if (so == 2) s->opts.use_graph = 0;   // host-driven loops cannot be captured
-    if (!res_wanted(s)) s->chain = chain_rule(s->opts, N, nnz);
   }
+  ResSetup R;
+  rc = plan_resident(s, H, h_sptr, h_sw, &R);
+  if (rc != BD_OK) {
+    std::string m = s->err;
+    release(s);
+    delete s;
+    return fail(nullptr, rc, "%s", m.c_str());
+  }
+  if (!R.fits) s->chain = chain_rule(s->opts, N, nnz);
   if (ok && (s->streaming || s->chain.one || s->chain.two)) {
     stream_prepare();   // kernel occupancies, queried outside any capture
     ok = alloc_n(s, reinterpret_cast<char**>(&s->d_sc), int64_t(2 * sizeof(StreamScal))) &&
@@ -2407,10 +2428,8 @@ int bd_create(const bd_mesh_t* mesh, const bd_cond_t* cond, bd_ionic_t model, co
     delete s;
     return fail(nullptr, BD_ERR_CUDA, "FP32 operator copy failed");
   }
-  AmgHost AH;
-  bool built = false;
-  rc = setup_resident(s, H, h_sptr, h_sw, &AH, &built);
-  if (rc == BD_OK && s->opts.elliptic_precond == 1) rc = setup_amg(s, H, AH, built);
+  rc = setup_resident(s, R);
+  if (rc == BD_OK && s->opts.elliptic_precond == 1) rc = setup_amg(s, H, R.AH);
   if (rc != BD_OK) {
     std::string m = s->err;
     release(s);

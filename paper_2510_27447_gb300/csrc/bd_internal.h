@@ -291,6 +291,9 @@ struct AmgHost {
   std::vector<double> cinv;        // dense inverse of A_c + c 1 1^T (nc x nc, row-major)
 };
 int amg_build(const HCsr& A, const AmgParams& prm, AmgHost* out, std::string* err);
+// drop levels so that H is what amg_build gives with a larger coarse_max (H must
+// have more than coarse_max rows on its finest level)
+int amg_truncate(int64_t coarse_max, AmgHost* H, std::string* err);
 
 struct SellHost {
   int64_t n = 0;

@@ -14,7 +14,8 @@ constexpr int kResMaxCluster = 16;    // blocks of a cluster (non-portable size)
 constexpr int kResBlock = 512;        // threads per block the kernels are built for (128 registers each)
 constexpr int kResMaxRows = 4;        // level-0 rows a thread may own
 constexpr int kResLevels = 5;         // smoothed levels the kernels can hold
-constexpr int kResCoarseMax = 384;    // rows of the dense coarsest level by default (see amg_params_resident)
+constexpr int kResSmemMax = 227 * 1024;   // shared memory a block may have
+constexpr int kResCoarseMax = 384;    // rows of the dense coarsest level by default (see plan_resident)
 
 // An operator's rows of one block, in the block's shared-memory image
 // (offsets in bytes from the image's start).  Rows are dealt 32 / g to a warp
