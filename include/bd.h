@@ -204,8 +204,10 @@ typedef struct {
                               registers); 2: as 0, with the mixed AMG kernels built for two
                               1024-thread blocks per SM (32 registers; operators of >= 12M
                               entries) */
-  int64_t amg_levels;      /* smoothed AMG levels of the elliptic preconditioner (0: Jacobi) */
-  int64_t amg_coarse_rows; /* rows of the dense coarsest AMG level (0: Jacobi) */
+  int64_t amg_levels;      /* smoothed AMG levels of the elliptic preconditioner (0: Jacobi; also 0
+                              for meshes of at most amg_coarse_max rows, whose mixed-precision
+                              cluster solves have a hierarchy of their own all the same) */
+  int64_t amg_coarse_rows; /* rows of the dense coarsest AMG level (0 where amg_levels is) */
   int64_t streaming;       /* 1: a streaming handle, 0: a persistent one (bd_opts_t.streaming) */
 } bd_stats_t;
 

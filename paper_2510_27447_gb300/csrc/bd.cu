@@ -142,7 +142,7 @@ struct bd_state {
   int mixed_grid = 1;
   int mixed_amg_grid = 1;                  // grid of the mixed AMG kernels (differs in tier 2)
   int amg_grid = 1;
-  int amg_levels = 0;
+  int amg_levels = 0, amg_coarse_rows = 0;   // of the hierarchy that preconditions, wherever it is held
   std::vector<int64_t> amg_shape;   // per level: rows, entries, form of A, R, P (bd_amg_level)
   double amg_cycle_bytes[2] = {0.0, 0.0};   // algorithmic bytes of one V-cycle's smoothed levels (FP64, FP32)
   double amg_cycle_opbytes[2] = {0.0, 0.0}; // ... of which operator values and indices
@@ -948,13 +948,43 @@ int setup_resident(bd_state* s, const ResSetup& R) {
   return BD_OK;
 }
 
+// algorithmic bytes of one V-cycle of the hierarchy (bd_profile_t), and the counts that
+// the statistics report
+void count_amg(bd_state* s, const AmgHost& AH) {
+  for (int v = 0; v < 2; ++v) {
+    const double vb = v == 0 ? 8.0 : 4.0;
+    double b = 0.0, ob = 0.0;
+    for (size_t l = 0; l < AH.lev.size(); ++l) {
+      const AmgHostLevel& Lh = AH.lev[l];
+      const double n = double(Lh.A.n), nn = double(Lh.P.m);
+      ob += double(2 * Lh.A.ci.size() + Lh.R.ci.size() + Lh.P.ci.size()) * (vb + 4);
+      // one product y = B x: (vb + 4) per entry, gather of x + result + row pointer per row
+      const double spA = double(Lh.A.ci.size()) * (vb + 4) + n * (2 * vb + 4);
+      const double spR = double(Lh.R.ci.size()) * (vb + 4) + nn * (vb + 4) + n * vb;
+      const double spP = double(Lh.P.ci.size()) * (vb + 4) + n * (vb + 4) + nn * vb;
+      // 2 A products (residual, post-smoothing), R, P; vector streams of the
+      // pre-smoothing (b, 1/D in, x out), residual (b in), prolongation (x in
+      // and out) and post-smoothing (b, 1/D in, y out)
+      b += 2 * spA + spR + spP + vb * (3 * n + n + 2 * n + 3 * n);
+    }
+    const double nc = double(AH.nc);
+    s->amg_cycle_bytes[v] = b;
+    s->amg_coarse_bytes[v] = vb * (nc * nc + 2 * nc);
+    s->amg_cycle_opbytes[v] = ob + vb * nc * nc;
+  }
+  s->amg_levels = int(AH.lev.size());
+  s->amg_coarse_rows = int(AH.nc);
+}
+
 // build the AMG hierarchy of A_ie on the host and upload it (SELL-32 operators)
-// (AH: the hierarchy planned for the cluster-resident solves, if any; kept when
-// they are taken, else its levels down to this one's coarsest)
+// (AH: the hierarchy planned for the cluster-resident solves, if any.  Where they
+// are taken it is theirs, and only its counts and shapes are kept here; else its
+// levels down to this one's coarsest)
 int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH) {
   std::string err;
   AmgParams prm;
   if (s->opts.amg_coarse_max > 0) prm.coarse_max = s->opts.amg_coarse_max;
+  if (s->res_amg) count_amg(s, AH);
   if (s->N <= prm.coarse_max) return BD_OK;   // small operator: Jacobi-PCG is used
   if (!s->res_on) {
     const int rc = AH.lev.empty() ? amg_build(elliptic_csr(s, H), prm, &AH, &err) : amg_truncate(prm.coarse_max, &AH, &err);
@@ -963,19 +993,37 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH) {
   if (AH.lev.empty()) return BD_OK;   // small operator: Jacobi-PCG is used
   if (int(AH.lev.size()) > kMaxAmgLevels)
     return fail(s, BD_ERR_ARG, "AMG hierarchy has %d levels", int(AH.lev.size()));
+  s->amg_shape.assign(AH.lev.size() * 9, 0);
+  // rows, entries and storage form (0 SELL-32, -1 wide SELL-32, k > 0 CSR
+  // with k lanes per row) of one operator of the hierarchy
+  auto shape = [&](size_t l, int which, const HCsr& M, bool csr, int lanes, int wmax) {
+    int64_t* o = s->amg_shape.data() + l * 9 + 3 * which;
+    o[0] = M.n;
+    o[1] = int64_t(M.ci.size());
+    o[2] = csr ? lanes : (wmax == 0 ? -1 : 0);
+  };
+  auto lanes_of = [&](const SellHost& S) {
+    const bool f64 = s->precision == BD_FP64;
+    return S.rp.empty() ? 0 : s->opts.csr_lanes > 0 ? s->opts.csr_lanes : csr_lanes(S.rp.back(), S.n, f64);
+  };
+  if (s->res_on) {   // the grid kernels' storage forms of the same operators
+    for (size_t l = 0; l < AH.lev.size(); ++l) {
+      const HCsr* const op[3] = {&AH.lev[l].A, &AH.lev[l].R, &AH.lev[l].P};
+      for (int k = 0; k < 3; ++k) {
+        if (l == 0 && k == 0) {
+          shape(l, k, *op[k], false, 0, s->wmax);
+          continue;
+        }
+        const SellHost S = sell_from_csr(*op[k], 0);
+        shape(l, k, *op[k], !S.rp.empty(), lanes_of(S), S.wmax);
+      }
+    }
+    return BD_OK;
+  }
   auto upload = [&](const void* h, size_t bytes) -> void* {
     void* d = dalloc(s, bytes);
     if (d && cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, s->stream) != cudaSuccess) return nullptr;
     return d;
-  };
-  s->amg_shape.assign(AH.lev.size() * 9, 0);
-  // rows, entries and storage form (0 SELL-32, -1 wide SELL-32, k > 0 CSR
-  // with k lanes per row) of one operator of the hierarchy
-  auto shape = [&](size_t l, int which, const HCsr& M, const SellDev& d) {
-    int64_t* o = s->amg_shape.data() + l * 9 + 3 * which;
-    o[0] = M.n;
-    o[1] = int64_t(M.ci.size());
-    o[2] = d.rp ? d.lpr : (d.wmax == 0 ? -1 : 0);
   };
   auto sell_dev = [&](const HCsr& M, SellDev* out) {
     const SellHost S = sell_from_csr(M, s->streaming ? s->opts.wide_sell + 1 : 0);
@@ -983,8 +1031,7 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH) {
     out->wmax = S.wmax;
     const bool csr = !S.rp.empty();
     out->rp = csr ? static_cast<const int64_t*>(upload(S.rp.data(), S.rp.size() * 8)) : nullptr;
-    const bool f64 = s->precision == BD_FP64;
-    out->lpr = csr ? (s->opts.csr_lanes > 0 ? s->opts.csr_lanes : csr_lanes(S.rp.back(), S.n, f64)) : 0;
+    out->lpr = lanes_of(S);
     out->sptr = csr ? nullptr : static_cast<const int64_t*>(upload(S.sptr.data(), S.sptr.size() * 8));
     out->sw = csr ? nullptr : static_cast<const int*>(upload(S.sw.data(), S.sw.size() * 4));
     out->col = static_cast<const int*>(upload(S.col.data(), S.col.size() * 4));
@@ -1006,9 +1053,9 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH) {
     }
     ok = ok && sell_dev(Lh.P, &Ld.P) && sell_dev(Lh.R, &Ld.R);
     if (ok) {
-      shape(size_t(l), 0, Lh.A, Ld.A);
-      shape(size_t(l), 1, Lh.R, Ld.R);
-      shape(size_t(l), 2, Lh.P, Ld.P);
+      shape(size_t(l), 0, Lh.A, Ld.A.rp != nullptr, Ld.A.lpr, Ld.A.wmax);
+      shape(size_t(l), 1, Lh.R, Ld.R.rp != nullptr, Ld.R.lpr, Ld.R.wmax);
+      shape(size_t(l), 2, Lh.P, Ld.P.rp != nullptr, Ld.P.lpr, Ld.P.wmax);
     }
     Ld.invd = static_cast<const double*>(upload(Lh.invdiag.data(), Lh.invdiag.size() * 8));
     Ld.omega = Lh.omega;
@@ -1128,28 +1175,7 @@ int setup_amg(bd_state* s, const HostOps& H, AmgHost& AH) {
   const int mx = pcg_amg_max_blocks(s->pcg_block, s->tier);
   if (mx <= 0) return fail(s, BD_ERR_CUDA, "cannot size the cooperative AMG-CG grid");
   s->amg_grid = std::min(s->pcg_grid, mx);
-  for (int v = 0; v < 2; ++v) {
-    const double vb = v == 0 ? 8.0 : 4.0;
-    double b = 0.0, ob = 0.0;
-    for (size_t l = 0; l < AH.lev.size(); ++l) {
-      const AmgHostLevel& Lh = AH.lev[l];
-      const double n = double(Lh.A.n), nn = double(Lh.P.m);
-      ob += double(2 * Lh.A.ci.size() + Lh.R.ci.size() + Lh.P.ci.size()) * (vb + 4);
-      // one product y = B x: (vb + 4) per entry, gather of x + result + row pointer per row
-      const double spA = double(Lh.A.ci.size()) * (vb + 4) + n * (2 * vb + 4);
-      const double spR = double(Lh.R.ci.size()) * (vb + 4) + nn * (vb + 4) + n * vb;
-      const double spP = double(Lh.P.ci.size()) * (vb + 4) + n * (vb + 4) + nn * vb;
-      // 2 A products (residual, post-smoothing), R, P; vector streams of the
-      // pre-smoothing (b, 1/D in, x out), residual (b in), prolongation (x in
-      // and out) and post-smoothing (b, 1/D in, y out)
-      b += 2 * spA + spR + spP + vb * (3 * n + n + 2 * n + 3 * n);
-    }
-    const double nc = double(AH.nc);
-    s->amg_cycle_bytes[v] = b;
-    s->amg_coarse_bytes[v] = vb * (nc * nc + 2 * nc);
-    s->amg_cycle_opbytes[v] = ob + vb * nc * nc;
-  }
-  s->amg_levels = M.nlev;
+  count_amg(s, AH);
   // the kernels read the descriptors from device memory
   if (cudaMemcpyAsync(s->d_amg, &s->amg, sizeof(AmgDev), cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
       cudaMemcpyAsync(s->d_amgf, &s->amgf, sizeof(AmgDevF), cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
@@ -2896,8 +2922,9 @@ int bd_get_stats(const bd_state_t* cs, bd_stats_t* out) {
   out->kernel_launches = s->launches + st[8];   // host-enqueued + counted on the device (streaming solves)
   out->solver_block_bound = s->cluster > 0 ? kSolverTierBlock[0] : kSolverTierBlock[s->tier];
   out->solver_tier = s->cluster > 0 ? 0 : s->tier;
-  out->amg_levels = s->use_amg ? s->amg.nlev : 0;
-  out->amg_coarse_rows = s->use_amg ? s->amg.nc : 0;
+  const bool levels = !s->amg_shape.empty();
+  out->amg_levels = levels ? s->amg_levels : 0;
+  out->amg_coarse_rows = levels ? s->amg_coarse_rows : 0;
   out->streaming = s->streaming ? 1 : 0;
   return BD_OK;
 }
@@ -3015,6 +3042,7 @@ int bd_profile_steps(bd_state_t* s, double dt, int M, int K, int n_steps, bd_pro
   out->outer_iters[1] = st1[5] - st0[5];
   // algorithmic bytes (see bd_profile_t); vb = bytes per value of the Krylov iteration
   const bool mixed = s->precision == BD_MIXED;
+  const bool amg = s->use_amg || s->res_amg;
   const double vb = mixed ? 4.0 : 8.0;
   const double pairs = double(st1[7] - st0[7]);     // two-RHS iterations in which both systems advanced
   const double pairs64 = double(st1[9] - st0[9]);   // FP64 operator passes shared by a streaming pair
@@ -3026,7 +3054,7 @@ int bd_profile_steps(bd_state_t* s, double dt, int M, int K, int n_steps, bd_pro
     auto spmv = [&](double v) { return nnz * (v + 4) + n * (2 * v + 4); };
     const double iters = double(out->cg_iters[k]), solves = double(out->cg_solves[k]);
     const double extra = ell ? 0.0 : 8.0 * n;                        // condensed diagonal
-    const double vec = (ell && s->use_amg ? 13.0 : 16.0) * vb * n;   // dots, axpys, (Jacobi)
+    const double vec = (ell && amg ? 13.0 : 16.0) * vb * n;   // dots, axpys, (Jacobi)
     const double per_iter = spmv(vb) + vec + extra;
     // per solve: right-hand-side products (elliptic A_i v; parabolic A_i a, M b, rl),
     // the set-up passes (rhs, 1/D, x, r) and, elliptic, projection and pin shift
@@ -3038,11 +3066,11 @@ int bd_profile_steps(bd_state_t* s, double dt, int M, int K, int n_steps, bd_pro
       // r32 and d32 out) and the update x += s d (x in and out, d in)
       b += outer * ((ell ? spmv(8.0) + 3.0 * 8.0 * n : 2.0 * 8.0 * n) + 16.0 * n + 20.0 * n);
     }
-    if (ell && s->use_amg) b -= pairs * nnz * (vb + 4);            // shared operator pass
+    if (ell && amg) b -= pairs * nnz * (vb + 4);            // shared operator pass
     if (ell) b -= pairs64 * nnz * (8.0 + 4.0);                     // shared FP64 products (A_i, A_ie)
     out->alg_bytes[k] = b;
   }
-  if (s->use_amg) {
+  if (amg) {
     const int v = mixed ? 1 : 0;
     // one cycle per iteration plus the first of each inner solve (mixed: every
     // refinement pass but the last, converged one of each solve)
@@ -3050,7 +3078,7 @@ int bd_profile_steps(bd_state_t* s, double dt, int M, int K, int n_steps, bd_pro
                           double(mixed ? out->outer_iters[0] - out->cg_solves[0] : out->cg_solves[0]);
     out->vcycle_bytes = cycles * s->amg_cycle_bytes[v];
     out->coarse_bytes = cycles * s->amg_coarse_bytes[v];
-    const double ncc = vb * double(s->amg.nc) * double(s->amg.nc);   // the dense coarse inverse
+    const double ncc = vb * double(s->amg_coarse_rows) * double(s->amg_coarse_rows);   // the dense coarse inverse
     out->vcycle_bytes -= (pairs + pairsc) * (s->amg_cycle_opbytes[v] - ncc);
     if (s->streaming || s->chain.two) out->coarse_bytes -= (pairs + pairsc) * ncc;   // read once for both systems
   }
