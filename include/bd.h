@@ -179,7 +179,8 @@ typedef struct {
                             passes serve both right-hand sides -- in mixed precision one
                             cooperative kernel (persistent form) or one kernel chain
                             (streaming form), in FP64 one kernel chain (streaming form; the
-                            persistent FP64 form solves one after the other).  0 (default):
+                            persistent FP64 form solves one after the other); cluster
+                            solves run as two clusters of one launch.  0 (default):
                             on; -1: one solve after the other (each
                             system's arithmetic is the same either way; the reductions are
                             formed over different block partitions); BD_ERR_ARG otherwise */

@@ -643,7 +643,7 @@ int elliptic(bd_state* s, const double* v, double* u) {
 // two solves
 int elliptic2(bd_state* s, const double* v1, double* u1, const double* v2, double* u2) {
   const bool mixed = s->precision == BD_MIXED;
-  if (s->res_on) {   // two clusters of one launch
+  if (s->res_on && s->opts.pair_solve >= 0) {   // two clusters of one launch
     if (s->NT < s->N) {
       Timed t(s, BD_K_COMBINE, 2);
       const int* gate = s->opts.sweep_tol > 0 ? s->gate : nullptr;
@@ -1872,7 +1872,7 @@ int enqueue_batch_step(BatchPlan& B, double dt, int M, int K) {
   // both elliptic constraints of a later sweep (M = 3) at once, for batches
   // whose solves are all cluster-resident and need no zero-padded potentials
   bool pairs = M == 3;
-  for (bd_state* s : B.m) pairs = pairs && s->res_on && s->NT == s->N;
+  for (bd_state* s : B.m) pairs = pairs && s->res_on && s->opts.pair_solve >= 0 && s->NT == s->N;
   auto elliptic_pairs = [&]() -> int {
     BatchSolveArgs q{};
     q.elliptic = true;
