@@ -267,7 +267,7 @@ bool dense_spd_inverse(std::vector<double>& a, int64_t n, std::vector<double>* i
 // the coarsest level of a hierarchy: dense inverse of A_c + c 1 1^T
 int coarse_inverse(const HCsr& A, AmgHost* out, std::string* err) {
   const int64_t n = A.n;
-  if (n > 4096) {
+  if (n > kDenseMax) {
     *err = "AMG: coarsest level too large for a dense solve";
     return BD_ERR_ARG;
   }

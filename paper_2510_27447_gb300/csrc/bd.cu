@@ -865,6 +865,46 @@ HCsr elliptic_csr(const bd_state* s, const HostOps& H) {
   return A;
 }
 
+constexpr int64_t kResMaxBytes = int64_t(kResMaxCluster) * 60 * 1024;   // see res_wanted
+
+// Is A_ie positive semi-definite with the constants as its only null vectors?
+// It is for positive conductivities on a connected mesh (every element matrix is
+// semi-definite with the constants as null space).
+bool surely_definite(const bd_state* s, const bd_cond_t* cond, const HostOps& H) {
+  if (!(cond->sil + cond->sel > 0.0) || !(cond->sit + cond->set > 0.0)) return false;
+  std::vector<uint8_t> seen(s->N, 0);
+  std::vector<int32_t> todo{0};
+  int64_t n = 1;
+  seen[0] = 1;
+  while (!todo.empty()) {
+    const int32_t i = todo.back();
+    todo.pop_back();
+    for (int64_t p = H.rowptr[i]; p < H.rowptr[i + 1]; ++p)
+      if (!seen[H.col[p]]) {
+        seen[H.col[p]] = 1;
+        ++n;
+        todo.push_back(H.col[p]);
+      }
+  }
+  return n == s->N;
+}
+
+// The meshes that the preconditioner refuses (a coarsest level that is too large
+// or not positive definite) are the same for every solver form and hierarchy:
+// where the outcome is not certain, the hierarchy of the options is built for it.
+int check_elliptic(bd_state* s, const bd_cond_t* cond, const HostOps& H) {
+  if (s->opts.elliptic_precond != 1) return BD_OK;
+  AmgParams prm;
+  if (s->opts.amg_coarse_max > 0) prm.coarse_max = s->opts.amg_coarse_max;
+  // larger meshes than a cluster holds have that hierarchy and no other
+  if (s->N > prm.coarse_max && s->nnz * 6 > kResMaxBytes) return BD_OK;
+  if (surely_definite(s, cond, H) && (s->N > prm.coarse_max || s->N <= kDenseMax)) return BD_OK;
+  AmgHost AH;
+  std::string err;
+  const int rc = amg_build(elliptic_csr(s, H), prm, &AH, &err);
+  return rc == BD_OK ? rc : fail(s, rc, "%s", err.c_str());
+}
+
 // may the handle's solves be cluster-resident?  Small problems whose solver
 // options are the defaults (forced tiers, grids, clusters and the streaming
 // form ask for the other kernels).  The plan decides whether it fits; an
@@ -873,7 +913,7 @@ HCsr elliptic_csr(const bd_state* s, const HostOps& H) {
 bool res_wanted(const bd_state* s) {
   const int64_t entry = s->precision == BD_MIXED ? 6 : 10;   // value and 16-bit column
   return !s->streaming && s->opts.cg_cluster == 0 && s->opts.solver_tier == 0 && s->opts.cg_block == 0 &&
-         s->opts.cg_grid == 0 && s->nnz * entry <= int64_t(kResMaxCluster) * 60 * 1024;
+         s->opts.cg_grid == 0 && s->nnz * entry <= kResMaxBytes;
 }
 
 // the cluster-resident solves' host plan and hierarchy
@@ -890,17 +930,19 @@ struct ResSetup {
 // precision also for meshes of fewer than 1500 rows.  FP64 solves of those keep
 // Jacobi: the tolerance bounds the residual, and another preconditioner would
 // move u by as much as it allows (1e-9 of u at the default 1e-10).
-int plan_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sptr, const std::vector<int>& sw,
-                  ResSetup* R) {
-  if (!res_wanted(s)) return BD_OK;
+void plan_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& sptr, const std::vector<int>& sw,
+                   ResSetup* R) {
+  if (!res_wanted(s)) return;
   const bool mixed = s->precision == BD_MIXED;
   AmgParams prm;
   if (s->opts.amg_coarse_max > 0) prm.coarse_max = s->opts.amg_coarse_max;
   else if (mixed || s->N > prm.coarse_max) prm.coarse_max = kResCoarseMax;
   if (s->opts.elliptic_precond == 1) {
     std::string err;
-    const int rc = amg_build(elliptic_csr(s, H), prm, &R->AH, &err);
-    if (rc != BD_OK) return fail(s, rc, "%s", err.c_str());
+    if (amg_build(elliptic_csr(s, H), prm, &R->AH, &err) != BD_OK) {   // setup_amg decides with its own hierarchy
+      R->AH = AmgHost{};
+      return;
+    }
   }
   R->amg = !R->AH.lev.empty();
   // the largest cluster the device schedules (a smaller one holds more per
@@ -913,7 +955,6 @@ int plan_resident(bd_state* s, const HostOps& H, const std::vector<int64_t>& spt
       break;
     R->fits = res_prepare(R->P.s, mixed, false) && (!R->amg || res_prepare(R->P.s, mixed, true));
   }
-  return BD_OK;
 }
 
 // upload the plan; every solve of the handle takes it from here on
@@ -2156,6 +2197,12 @@ int bd_create(const bd_mesh_t* mesh, const bd_cond_t* cond, bd_ionic_t model, co
     delete s;
     return fail(nullptr, BD_ERR_ARG, "pin_node out of range");
   }
+  rc = check_elliptic(s, cond, H);
+  if (rc != BD_OK) {
+    std::string m = s->err;
+    delete s;
+    return fail(nullptr, rc, "%s", m.c_str());
+  }
   // SELL-32 layout of the shared pattern
   const int64_t nsl = (s->N + 31) / 32;
   std::vector<int64_t> h_sptr(nsl);
@@ -2319,13 +2366,7 @@ int bd_create(const bd_mesh_t* mesh, const bd_cond_t* cond, bd_ionic_t model, co
     if (so == 2) s->opts.use_graph = 0;   // host-driven loops cannot be captured
   }
   ResSetup R;
-  rc = plan_resident(s, H, h_sptr, h_sw, &R);
-  if (rc != BD_OK) {
-    std::string m = s->err;
-    release(s);
-    delete s;
-    return fail(nullptr, rc, "%s", m.c_str());
-  }
+  plan_resident(s, H, h_sptr, h_sw, &R);
   if (!R.fits) s->chain = chain_rule(s->opts, N, nnz);
   if (ok && (s->streaming || s->chain.one || s->chain.two)) {
     stream_prepare();   // kernel occupancies, queried outside any capture

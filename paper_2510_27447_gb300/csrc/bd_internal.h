@@ -275,6 +275,7 @@ struct HCsr {                      // host CSR, n x m
   std::vector<int32_t> ci;
   std::vector<double> v;
 };
+constexpr int64_t kDenseMax = 4096;   // rows of a dense coarsest level, at most
 struct AmgParams {
   double theta = 0.08;             // strength-of-connection threshold
   int64_t coarse_max = 1500;       // rows of the dense coarsest solve
