@@ -26,9 +26,9 @@
 // and two mbarriers in turn (SumTurns), and so do the halos that travel with
 // them in the pipelined loop.
 //   Waits for peers are bounded (kWaitLimitNs).  On expiry a warp records
-// ST_TIMEOUT; the block's next barrier tells all its warps, which then leave
-// through the cluster barrier at the kernel's end, so that no block is gone
-// while a peer may still send to it (PhaseOrder).
+// ST_TIMEOUT; the block's next barrier tells all its warps, which then end, except
+// the first, which leaves through the cluster barrier at the kernel's end, so
+// that no block is gone while a peer may still send to it (PhaseOrder).
 //
 // The iteration is the one of the grid kernels: Jacobi- or AMG-V(1,1)-
 // preconditioned CG; T = double solves in FP64, T = float is the mixed path's
@@ -158,6 +158,9 @@ struct PhaseHw {
     asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(gone) : "r"(flag) : "memory");
     return gone;
   }
+  __device__ __forceinline__ void end_unless_first() const {
+    if (threadIdx.x >= 32) asm volatile("exit;");
+  }
   // the block expects bytes from its peers in phase k (thread 0, after a
   // barrier of the block behind the phase's own work)
   __device__ __forceinline__ void expect(int k, int bytes) const {
@@ -215,7 +218,6 @@ using Phases = PhaseOrder<PhaseHw>;
 // the block's own halo (bytes: what the block expects in phase k besides)
 template <class T>
 __device__ __forceinline__ void exchange(Phases& ph, const uint32_t* word, int n, T* vec, int k, int bytes) {
-  if (!ph.ok()) return;
   const int gone = ph.meet();
   ph.expect(k, bytes);
 #pragma unroll 1
@@ -229,7 +231,6 @@ __device__ __forceinline__ void exchange(Phases& ph, const uint32_t* word, int n
 // count values of a coarse vector, owned from c0 on (a multiple of 4), to every block
 template <class T>
 __device__ __forceinline__ void gather_all(Phases& ph, T* vec, int c0, int count, int C, int k, int bytes) {
-  if (!ph.ok()) return;
   const int gone = ph.meet();
   ph.expect(k, bytes);
   const int sh = 31 - __clz(C);          // C is a power of two
@@ -298,9 +299,10 @@ __device__ __forceinline__ void op_rows(const ResOp& o, const unsigned char* img
 // FP64 sums over the cluster: through shared memory to four warps (whose lanes
 // all add distinct values, see sparse.cuh:block_sum), their partials to every
 // block; thread 0 adds the totals and runs f(totals), which writes shared
-// variables the block reads afterwards.
+// variables the block reads afterwards.  Returns what the last barrier brought,
+// for learn() (the caller's reads of those variables may go ahead of it).
 template <int NV, class F>
-__device__ __forceinline__ void sum_f64(Phases& ph, int k, int part_slot, double (&v)[NV], double* stage, double* part,
+__device__ __forceinline__ int sum_f64(Phases& ph, int k, int part_slot, double (&v)[NV], double* stage, double* part,
                                         int C, int rank, F&& f) {
   static_assert(NV <= 3, "up to three values");
   constexpr int G = NV == 1 ? 32 : NV == 2 ? 16 : 8;   // lanes that end with one value
@@ -308,7 +310,6 @@ __device__ __forceinline__ void sum_f64(Phases& ph, int k, int part_slot, double
   double* pt = part + part_slot * 3 * 4 * kResMaxCluster;
 #pragma unroll
   for (int i = 0; i < NV; ++i) stage[i * bd + threadIdx.x] = v[i];
-  if (!ph.ok()) return;
   const int gone = ph.meet();
   ph.expect(k, C * 4 * NV * 8);
   if (wid < 4) {
@@ -337,7 +338,7 @@ __device__ __forceinline__ void sum_f64(Phases& ph, int k, int part_slot, double
     for (int i = 0; i < NV; ++i) p[i] = __shfl_sync(0xffffffffu, x, i * G);
     if (lane == 0 && !ph.late()) f(p);
   }
-  ph.sync();
+  return ph.meet();
 }
 
 // FP32 sums of three values over the cluster: every warp sends its partials
@@ -563,7 +564,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
   };
   {
     const int k = next_sum();
-    sum_f64<2>(ph, k, k - kSum0, s2, stage, partd, iC, irank, [&](const double (&t)[2]) {
+    ph.learn(sum_f64<2>(ph, k, k - kSum0, s2, stage, partd, iC, irank, [&](const double (&t)[2]) {
       double bb = t[1];
       s_d[0] = 0.0;
       if (a.project) {
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
       s_d[1] = bb;
       s_d[2] = a.tol * a.tol * bb;
       if (!a.project) decide(t[0]);
-    });
+    }));
   }
   if (a.project) {
     const double mean = s_d[0];
@@ -587,7 +588,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
         s1[0] += r64[j] * r64[j];
       }
     const int k = next_sum();
-    sum_f64<1>(ph, k, k - kSum0, s1, stage, partd, iC, irank, [&](const double (&t)[1]) { decide(t[0]); });
+    ph.learn(sum_f64<1>(ph, k, k - kSum0, s1, stage, partd, iC, irank, [&](const double (&t)[1]) { decide(t[0]); }));
   }
 
   int fail = 0;
@@ -610,7 +611,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
           s1[0] += r64[j] * r64[j];
         }
       const int k = next_sum();
-      sum_f64<1>(ph, k, k - kSum0, s1, stage, partd, iC, irank, [&](const double (&t)[1]) { decide(t[0]); });
+      ph.learn(sum_f64<1>(ph, k, k - kSum0, s1, stage, partd, iC, irank, [&](const double (&t)[1]) { decide(t[0]); }));
     }
     if (!ph.ok()) break;
     const int code = s_code;
@@ -847,7 +848,6 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
         if (!first) ++it;
         if constexpr (F32) {
           const int turn = turns32.next(), k = kRed + turn;
-          if (!ph.ok()) break;
           const int gone = ph.meet();   // the products' vector is read
           ph.expect(k, nparts * 16);
           sum_f32_send(ph, k, turn, t3, partf, iC, irank, nw);
@@ -881,7 +881,7 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
           double (&td)[3] = reinterpret_cast<double (&)[3]>(t3);
           // s_code: 0 go on, -1 converged, else the failure
           const int k = next_sum();
-          sum_f64<3>(ph, k, k - kSum0, td, stage, partd, iC, irank, [&](const double (&t)[3]) {
+          const int gone = sum_f64<3>(ph, k, k - kSum0, td, stage, partd, iC, irank, [&](const double (&t)[3]) {
             s_code = first ? (!(t[2] > s_d[2]) ? -1 : 0)   // includes b = 0
                      : !isfinite(t[2]) || !isfinite(t[0]) ? ST_NONFINITE
                      : t[2] <= s_d[2]                     ? -1
@@ -896,13 +896,15 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
               rho = t[0];
             }
           });
-          if (!ph.ok()) break;
-          if (s_code != 0) {
-            fail = s_code > 0 ? s_code : 0;
-            break;
-          }
+          const int next = s_code;
           beta = s_d[4];
           alpha = s_d[3];
+          ph.learn(gone);
+          if (!ph.ok()) break;
+          if (next != 0) {
+            fail = next > 0 ? next : 0;
+            break;
+          }
         }
 #pragma unroll
         for (int j = 0; j < RPT; ++j) {
@@ -939,8 +941,8 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
     for (int j = 0; j < RPT; ++j)
       if (tid + j * bd < nloc) s1[0] += xs[j];
     const int k = next_sum();
-    sum_f64<1>(ph, k, k - kSum0, s1, stage, partd, iC, irank,
-               [&](const double (&t)[1]) { s_d[0] = t[0] / double(a.n); });
+    ph.learn(sum_f64<1>(ph, k, k - kSum0, s1, stage, partd, iC, irank,
+                        [&](const double (&t)[1]) { s_d[0] = t[0] / double(a.n); }));
     shift = s_d[0];
   }
   if (ph.sync()) {

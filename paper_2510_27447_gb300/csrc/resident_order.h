@@ -33,21 +33,24 @@ struct SumTurns {
 // solve goes on.  Hw::await(k, parity) waits for phase k of this block with a
 // limit and returns false when that has passed.  Hw::block_sync(late, turn) is
 // the block's barrier: a late warp sets the block's flag of this turn before it,
-// every warp returns that flag as it finds it behind it.
+// every warp returns that flag as it finds it behind it.  Hw::end_unless_first()
+// ends every warp but the block's first (ended warps count as arrived at all
+// barriers to come).
 //   A wait that has run out concerns its warp alone (the message may arrive
 // before another warp's limit), so nothing but late() follows from it there and
-// then.  At the block's next barrier every warp learns of it at once: ok() is the
-// same in the whole block, and a block that is not ok passes no further barrier.
-// (Two flags, for barriers in turn: with one, a warp whose next wait has run out
-// already could set it before a slow one has read what the barrier brought.)  A
-// late warp goes on to its next barrier, whichever that is, without waiting for
-// peers; every path of a solve has one (the one before its results are stored,
-// if no other).  So all warps of a block pass equally many barriers, and every
-// wait has an end.
+// then.  A late warp goes on to its next barrier, whichever that is, without
+// waiting for peers; every path of a solve has one (the one before its results
+// are stored, if no other).  There every warp of the block learns of it at once:
+// all end but the first, which meets no one at the block's further barriers,
+// waits for no phase and goes to the kernel's last barrier, so that the block
+// is there as long as a peer may send to it.  No warp is left waiting.
+//   (Two flags, for barriers in turn: with one, a warp whose next wait has run
+// out already could set it before a slow one has read what the barrier brought.)
 //   The flag is read with the barrier and used after the phase's sends (meet,
-// learn).  With a reducing barrier (__syncthreads_or) instead, measured on GB300,
-// a step against this form: TP06 129^2 mixed 1.88 / 1.83 ms, LR91 65^2 FP64 1.96 /
-// 1.92, a batch of twelve 3.43 / 3.35.
+// learn).  Measured on GB300, ms per step with a reducing barrier
+// (__syncthreads_or) whose outcome every phase waits for and tests / with this:
+// TP06 129^2 mixed 1.88 / 1.76, LR91 65^2 FP64 1.96 / 1.91, a batch of twelve 3.43 /
+// 3.30.
 template <class Hw>
 struct PhaseOrder : Hw {
   unsigned par = 0;      // parity of each phase's next completion, and three flags
@@ -56,17 +59,20 @@ struct PhaseOrder : Hw {
   // a wait of this warp has run out; no warp's had at the block's last barrier
   BD_ORDER_FN bool late() const { return (par & kLate) != 0u; }
   BD_ORDER_FN bool ok() const { return (par & kGone) == 0u; }
-  // barrier of a block that is ok; its outcome, for learn()
+  // the block's barrier; its outcome, for learn()
   BD_ORDER_FN int meet() {
     const int gone = Hw::block_sync(late(), (par & kTurn) != 0u);
     par ^= kTurn;
     return gone;
   }
   BD_ORDER_FN void learn(int gone) {
-    if (gone) par |= kGone;
+    if (gone) {
+      Hw::end_unless_first();
+      par |= kGone;
+    }
   }
   BD_ORDER_FN bool sync() {
-    if (ok()) learn(meet());
+    learn(meet());
     return ok();
   }
   BD_ORDER_FN void wait(int k) {

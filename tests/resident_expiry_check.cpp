@@ -2,7 +2,7 @@
 // four warps (threads here): PhaseOrder (resident_order.h) over barriers and
 // phases that count messages, and a script of messages that come late or never.
 // Every barrier of the model gives up after three seconds: a warp that meets
-// that limit would have hung.  Usage: resident_expiry_check rule script
+// that limit would have hung (so would a phase expected twice).  Usage: resident_expiry_check rule script
 //   rule    order   PhaseOrder
 //           alone   a late warp leaves by itself (the block's first to the cluster
 //                   barrier, the others end), which hangs in script "between"
@@ -65,6 +65,7 @@ struct Mb {
     std::lock_guard<std::mutex> l(m);
     arrivals += a;
     tx += t;
+    if (arrivals > 1) stuck = true;   // a phase expected again before it was complete
     if (arrivals == 1 && tx == 0) {
       arrivals = 0;
       ++done;
@@ -106,6 +107,10 @@ struct Hw {
     if (script.rfind("random", 0) == 0 && std::rand() % 16 == 0) std::this_thread::sleep_for(Ms(120));
     return b.flag[turn];
   }
+  struct Ended {};
+  void end_unless_first() const {
+    if (warp > 0) throw Ended{};
+  }
   bool await(int k, unsigned p) const {
     Mb& b = cl->blk[block].mb[k];
     std::unique_lock<std::mutex> l(b.m);
@@ -124,33 +129,37 @@ void send(int to, int k, int ms) {
   }).detach();
 }
 
-void warp(int block, int w, bool alone, unsigned seed) {
+void solve(int block, int w, bool alone, std::mt19937& g) {
   PhaseOrder<Hw> ph{{block, w}};
   SumTurns turns;
-  std::mt19937 g(seed);
-  bool gone = false;
-  for (int step = 0; step < kSteps && !gone; ++step) {
+  for (int step = 0; step < kSteps; ++step) {
     const int k = step % 2 ? kSum0 + turns.next() : int(kZ);   // as the Jacobi loop
-    if (!ph.ok()) break;
-    const int gone_now = ph.meet();
+    const int gone = ph.meet();
     if (w == 0) {
       cl->blk[block].mb[k].add(1, 1);
       send(1 - block, k, travel(block, step, g));
     }
-    ph.learn(gone_now);
+    ph.learn(gone);
     ph.wait(k);
     if (alone && ph.late()) {
-      if (w > 0) {
-        cl->blk[block].bar.leave();
-        cl->all.leave();
-        ++finished;
-        return;
-      }
-      gone = true;
+      if (w > 0) throw Hw::Ended{};
+      return;
     }
+    // the loop's test, once an iteration; a late warp may take another way at its decisions
+    if (step % 2 && (!ph.ok() || (ph.late() && w % 2))) break;
   }
   if (!alone) ph.sync();
-  cl->all.arrive();
+}
+
+void warp(int block, int w, bool alone, unsigned seed) {
+  std::mt19937 g(seed);
+  try {
+    solve(block, w, alone, g);
+    cl->all.arrive();
+  } catch (Hw::Ended&) {
+    cl->blk[block].bar.leave();
+    cl->all.leave();
+  }
   ++finished;
 }
 
