@@ -306,7 +306,8 @@ int bd_step_adaptive(bd_state_t* s, double dt_max, double tol, int n_sdc_nodes, 
 /* Failure-path check (the paper has no counterpart): one block waits at a
  * device-wide barrier sized for two blocks, so the wait runs out after its
  * bound of about two seconds of device time, as a solver's wait would if a
- * block never arrived.  Returns BD_ERR_TIMEOUT when the bound works (any
+ * block never arrived; then, on a handle whose solves run in one cluster, a
+ * block of a solve expects a message that nobody sends.  Returns BD_ERR_TIMEOUT when the bound works (any
  * other value is a fault of the build); the handle's status word and barrier
  * are reset afterwards, so the handle stays usable. */
 int bd_selftest_wait_timeout(bd_state_t* s);

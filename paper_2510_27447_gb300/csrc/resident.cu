@@ -47,12 +47,17 @@
 // problem takes the whole 16-block cluster however small it is, FP64 scalars
 // are formed by one thread, and sums are added by four warps a block.
 //
+// Registers: every instance is built for kResBlock threads, 128 registers each, and
+// the AMG instances spill (stores: FP32 0.6 to 1.7 KB, FP64 1.0 to 2.4 KB; pipelined
+// Jacobi 0.2 to 0.7 KB, FP64 Jacobi below 0.1), to L1; without opaque() it was more.
+// Instances built for the 128 to 416 threads that the plans ask for would spill less.
+//
 // Measured on GB300, ms per step (three nodes, two sweeps), grid kernels / one
-// cluster: LR91 33^2 mixed 4.13 / 0.62, LR91 65^2 FP64 6.45 / 2.02, TP06 129^2
-// mixed 2.75 / 1.87, LR91 101^2 FP64 adaptive 5.66 / 2.82 and CN-RK2 1.24 / 0.73,
-// a batch of twelve 65^2 and 129^2 requests (against streaming chains) 9.02 / 3.40.
-// Both sides at the largest sizes that fit: LR91 140^2 mixed 2.23 / 1.62, 115^2 FP64
-// 4.51 / 3.10, slab 25x25x8 FP64 5.58 / 2.79.
+// cluster: LR91 33^2 mixed 4.10 / 0.65, LR91 65^2 FP64 6.35 / 1.91, TP06 129^2
+// mixed 2.63 / 1.76, LR91 101^2 FP64 adaptive 5.66 / 2.73 and CN-RK2 1.20 / 0.68,
+// a batch of twelve 65^2 and 129^2 requests (against streaming chains) 9.23 / 3.30.
+// Both sides near the largest sizes that fit: LR91 119^2 mixed 2.12 / 1.20 and FP64
+// 5.28 / 2.88, slabs 30x30x8 mixed 2.63 / 1.42 and 25x25x8 FP64 5.58 / 2.79.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -142,6 +147,8 @@ __device__ __forceinline__ void cp_block(unsigned char* dst, const void* src, in
     cp_async16(d + i, static_cast<const unsigned char*>(src) + i);
 }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+constexpr unsigned long long kDrainNs = 1000000ull;
 
 // the block's mbarriers, its barrier and flags, as PhaseOrder uses them
 struct PhaseHw {
@@ -955,6 +962,12 @@ __global__ void __launch_bounds__(kResBlock, 1) res_kernel(const __grid_constant
     if (a.iters_acc) atomicAdd((unsigned long long*)a.iters_acc, (unsigned long long)inner_total);
     if (a.outer_acc && F32) atomicAdd((unsigned long long*)a.outer_acc, (unsigned long long)outer_total);
     if (a.solves_acc) atomicAdd((unsigned long long*)a.solves_acc, 1ull);
+  }
+  // after an expiry, messages of this block may still be on their way to blocks
+  // that wait for nothing any more; they land in a few microseconds
+  if (!ph.ok()) {
+    const unsigned long long t0 = device_ns();
+    for (int n = 0; n < 100000 && device_ns() - t0 < kDrainNs; ++n) __nanosleep(100);
   }
   __syncwarp();
   cluster_barrier();   // no block leaves while a peer may still send to it

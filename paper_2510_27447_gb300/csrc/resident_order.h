@@ -43,7 +43,9 @@ struct SumTurns {
 // are stored, if no other).  There every warp of the block learns of it at once:
 // all end but the first, which meets no one at the block's further barriers,
 // waits for no phase and goes to the kernel's last barrier, so that the block
-// is there as long as a peer may send to it.  No warp is left waiting.
+// is there as long as a peer may send to it (before that barrier it lets a
+// millisecond pass, in which what the block has sent arrives: a peer that has given
+// up does not wait for it).  No warp is left waiting.
 //   (Two flags, for barriers in turn: with one, a warp whose next wait has run
 // out already could set it before a slow one has read what the barrier brought.)
 //   The flag is read with the barrier and used after the phase's sends (meet,
